@@ -15,7 +15,9 @@ ROOT = os.path.dirname(PKG)
 CSRC = os.path.join(PKG, "csrc")
 LIBDIR = os.path.join(PKG, "_lib")
 OBJDIR = os.path.join(ROOT, "_build")
-SOURCES = ["host.cu", "ntt.cu", "kernels.cu", "ext.cu", "api.cu"]
+# (object, source, defines): ntt.cu's kernels compile as four objects in parallel
+UNITS = [("host", "host.cu", []), ("kernels", "kernels.cu", []), ("ext", "ext.cu", []), ("api", "api.cu", [])]
+UNITS += [("ntt%d" % p, "ntt.cu", ["-DBFHE_NTT_PART=%d" % p]) for p in range(4)]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC", "-Xcompiler", "-O2"]
 
@@ -45,11 +47,11 @@ def build(verbose=False, force=False):
     headers = [os.path.join(CSRC, h) for h in os.listdir(CSRC) if h.endswith((".cuh", ".h"))]
     headers.append(os.path.join(ROOT, "include", "bfhe.h"))
     jobs = []
-    for src in SOURCES:
+    for name, src, defs in UNITS:
         s = os.path.join(CSRC, src)
-        o = os.path.join(OBJDIR, src.replace(".cu", ".o"))
+        o = os.path.join(OBJDIR, name + ".o")
         if force or _stale(o, [s] + headers):
-            jobs.append([nvcc, *ARCH, *FLAGS, "-c", s, "-o", o])
+            jobs.append([nvcc, *ARCH, *FLAGS, *defs, "-c", s, "-o", o])
 
     def run(cmd):
         r = subprocess.run(cmd, capture_output=True, text=True)
@@ -58,9 +60,9 @@ def build(verbose=False, force=False):
         if verbose:
             sys.stdout.write(r.stdout + r.stderr)
 
-    with cf.ThreadPoolExecutor(max_workers=len(SOURCES)) as ex:
+    with cf.ThreadPoolExecutor(max_workers=len(UNITS)) as ex:
         list(ex.map(run, jobs))
-    objs = [os.path.join(OBJDIR, s.replace(".cu", ".o")) for s in SOURCES]
+    objs = [os.path.join(OBJDIR, name + ".o") for name, _, _ in UNITS]
     lib = lib_path()
     if force or jobs or _stale(lib, objs):
         tmp = lib + ".tmp"

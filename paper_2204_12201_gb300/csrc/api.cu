@@ -865,6 +865,7 @@ extern "C" int bfhe_ntt(bfhe_ctx* c, uint64_t* data, size_t n_polys, uint32_t n_
     if (!data || n_limbs == 0 || n_limbs > c->L) return set_error(BFHE_EINVAL, "bad arguments");
     if (n_polys == 0) return BFHE_OK;
     NttIO io = ntt_io(data, data, n_limbs, c->N);
+    io.natural = true;
     if (inverse) return launch_ntt_inv(c, io, (int)n_polys, (int)n_limbs, c->mapQ(), 0, S(stream));
     return launch_ntt_fwd(c, io, (int)n_polys, (int)n_limbs, c->mapQ(), S(stream));
 }

@@ -100,6 +100,77 @@ __host__ __device__ __forceinline__ u64 reduce64(u64 x, u64 q, u64 mu) {
     return r >= q ? r - q : r;
 }
 
+// ------------------------------------------------------------------ products modulo q = 2^b - d
+// The parameter rule scans downwards from 2^b, so every modulus is q = 2^b - d with d below 2^27, and 2^(b+2) = 4d
+// (mod q).  A product by a constant w takes the table entry e of w: with v = 2^32 w mod q and both cut at bit
+// k = b - 30, e.x = wl | wh << 32, e.y = vl | vh << 32 (wl, vl < 2^k; wh, vh < 2^30).  For a = a1 2^32 + a0 (a signed
+// 64-bit word, a0 its unsigned low half)
+//   a w = a0 w + a1 v = P + 2^k Q,   P = a0 wl + a1 vl,   Q = a0 wh + a1 vh = qh 2^32 + ql,
+//   pm_mul = P + 2^k ql + 4d qh,
+// signed, congruent to a w and below 3 2^29 4d + 2^(b+3.4) in magnitude for |a| < 2^63: five 32 x 32 -> 64-bit
+// multiply-adds and two shifts.  Shoup's product above takes five wide and four narrow ones; on this chip a wide
+// multiply holds the multiplier pipe four cycles per warp and scheduler, a narrow one or any other operation two, so the
+// pipe is the bound of every transform: 9.7 -> 7.0 SM cycles per warp butterfly (registers only, GB300).
+__device__ __forceinline__ u64 mad_wide_u(uint32_t a, uint32_t b, u64 c) {
+    // as a carry pair: one wide multiply-add (the 64-bit form compiles to a multiply, an add and a move)
+    uint32_t lo = (uint32_t)c, hi = (uint32_t)(c >> 32);
+    asm("mad.lo.cc.u32 %0, %2, %3, %0;\n\tmadc.hi.u32 %1, %2, %3, %1;" : "+r"(lo), "+r"(hi) : "r"(a), "r"(b));
+    return ((u64)hi << 32) | lo;
+}
+__device__ __forceinline__ u64 mad_wide_s(int a, int b, u64 c) {
+    uint32_t lo = (uint32_t)c, hi = (uint32_t)(c >> 32);
+    asm("mad.lo.cc.s32 %0, %2, %3, %0;\n\tmadc.hi.s32 %1, %2, %3, %1;" : "+r"(lo), "+r"(hi) : "r"(a), "r"(b));
+    return ((u64)hi << 32) | lo;
+}
+__device__ __forceinline__ u64 add64(u64 a, u64 b) {
+    uint32_t lo, hi;
+    asm("add.cc.u32 %0, %2, %4;\n\taddc.u32 %1, %3, %5;"
+        : "=r"(lo), "=r"(hi)
+        : "r"((uint32_t)a), "r"((uint32_t)(a >> 32)), "r"((uint32_t)b), "r"((uint32_t)(b >> 32)));
+    return ((u64)hi << 32) | lo;
+}
+__device__ __forceinline__ u64 sub64(u64 a, u64 b) {
+    uint32_t lo, hi;
+    asm("sub.cc.u32 %0, %2, %4;\n\tsubc.u32 %1, %3, %5;"
+        : "=r"(lo), "=r"(hi)
+        : "r"((uint32_t)a), "r"((uint32_t)(a >> 32)), "r"((uint32_t)b), "r"((uint32_t)(b >> 32)));
+    return ((u64)hi << 32) | lo;
+}
+__device__ __forceinline__ u64 pm_mul(u64 a, ulonglong2 e, int k, uint32_t d4) {
+    const uint32_t a0 = (uint32_t)a;
+    const int a1 = (int)(a >> 32);
+    u64 Q = (u64)a0 * (uint32_t)(e.x >> 32);
+    Q = mad_wide_s(a1, (int)(e.y >> 32), Q);
+    const uint32_t ql = (uint32_t)Q;
+    u64 T = ((u64)(ql >> (32 - k)) << 32) | (ql << k);
+    T = mad_wide_u(a0, (uint32_t)e.x, T);
+    T = mad_wide_s(a1, (int)(uint32_t)e.y, T);
+    return mad_wide_s((int)(Q >> 32), (int)d4, T);
+}
+// signed x = h 2^b + l (0 <= l < 2^b) to the congruent h d + l, above -2^(63-b) d and below 2^b + 2^(63-b) d
+__device__ __forceinline__ u64 pm_fold(u64 x, int b, uint32_t d) {
+    const int xh = (int)(x >> 32);
+    const u64 l = ((u64)((uint32_t)xh & ((1u << (b - 32)) - 1u)) << 32) | (uint32_t)x;
+    return mad_wide_s(xh >> (b - 32), (int)d, l);
+}
+// a signed 64-bit word to its residue below 2^b + 2^(63-b) d < 2q (non-negative)
+__device__ __forceinline__ u64 pm_lazy(u64 x, u64 q, int b, uint32_t d) {
+    const u64 y = pm_fold(x, b, d);
+    return add64(y, (u64)((i64)y >> 63) & q);
+}
+// to the canonical residue
+__device__ __forceinline__ u64 pm_canon(u64 x, u64 q, int b, uint32_t d) {
+    const u64 y = pm_lazy(x, q, b, d);
+    return y >= q ? y - q : y;
+}
+// host: the table entry of w
+inline void pm_entry(u64 w, u64 q, int b, u64* x, u64* y) {
+    const int k = b - 30;
+    const u64 m = ((u64)1 << k) - 1, v = (u64)(((u128)w << 32) % q);
+    *x = (w & m) | ((w >> k) << 32);
+    *y = (v & m) | ((v >> k) << 32);
+}
+
 // ------------------------------------------------------------------ exact base extension tables
 // Centred extension of an integer given by residues modulo the source primes
 // s_0..s_{n-1} (S = prod s_i) to target primes T_0..T_{m-1}: Garner's mixed
@@ -139,12 +210,13 @@ struct ExtHost {
 };
 
 // Device-side prime tables of a context, by prime index
-// (0..L-1 data, L..L+alpha-1 special, L+alpha..L+alpha+K-1 auxiliary, last: t).
+// (0..L-1 data, L..L+alpha-1 special, L+alpha..L+alpha+K-1 auxiliary, last: t).  The pairs of tw, twl, itw and
+// twist are pm_mul's entries for the moduli of a context with pm set, (w, Shoup(w)) otherwise and always for t.
 struct PrimeTab {
     const u64* q;        // modulus
     const u64* qinv;     // -q^-1 mod 2^64
     const u64* mu;       // floor(2^64 / q)
-    const u64* tw;       // [nP][N][2] (psi^brv(k), Shoup companion)      forward twiddles
+    const u64* tw;       // [nP][N][2] psi^brv(k)                         forward twiddles
     const u64* twl;      // [nP][3][N][2] the same, stages b < le regrouped per le = 3, 4, 5 (forward last pass)
     const u64* itw;      // [nP][N][2] inverse (DIT) twiddles: entry 2^b + j = omega^-(N/2^(b+1)) j, omega = psi^2
     const u64* twist;    // [nP][3][N][2] output twist N^-1 psi^-m (plain; times R = 2^64; times t R), mod q
@@ -161,6 +233,7 @@ struct bfhe_ctx {
     int device = 0;
     uint32_t N = 0, logN = 0, L = 0, alpha = 0, K = 0, nP = 0, prime_bits = 0;
     u64 t = 0;
+    bool pm = false;        // the moduli's products run as pm_mul: 45 to 55 bits, transforms bounded below 2^63
     bool batching = true;   // t = 1 mod 2N: slot encoding; t = 2: coefficient encoding only
     std::vector<u64> primes;     // nP: Q, P, B, t
     std::vector<uint32_t> brv;   // host copy of bit reversal (N)
@@ -168,7 +241,7 @@ struct bfhe_ctx {
     void* d_arena = nullptr;     // all constant tables
     size_t arena_bytes = 0;
     PrimeTab tab{};
-    uint32_t* d_brv = nullptr;   // [N]
+    uint32_t* d_brv = nullptr;   // [N] storage position of slot j's evaluation
     ExtDesc ext_QB{}, ext_BQ{}, ext_PQ{}, ext_Qt{};
     ExtHost exth_QB, exth_BQ;
     // Shoup pair tables: p[i] = w_i, p[n + i] = ws_i
@@ -223,6 +296,7 @@ struct bfhe_ctx {
     mutable std::vector<ProfRec> prof_pending;
     mutable std::vector<cudaEvent_t> prof_pool;
 
+    int pm_bits() const { return pm ? (int)prime_bits : 0; }
     LimbMap mapQ() const { return LimbMap{(int)L, 0}; }
     LimbMap mapQP() const { return LimbMap{(int)(L + alpha), 0}; }
     LimbMap mapQB() const { return LimbMap{(int)L, (int)alpha}; }
@@ -277,6 +351,7 @@ struct NttIO {
     int n_inner;
     size_t in_os, in_is, in_ls;
     size_t out_os, out_is, out_ls;
+    bool natural = false;   // the evaluation side in bit-reversed index order (bfhe_ntt) rather than the storage order
 };
 // contiguous [n_polys][n_limbs][N] in and out
 inline NttIO ntt_io(const u64* in, u64* out, size_t n_limbs, size_t N) {
@@ -289,15 +364,13 @@ inline NttIO ntt_io(const u64* in, u64* out, size_t n_limbs, size_t N) {
     io.in_ls = io.out_ls = N;
     return io;
 }
-// lazy_out: outputs left below 64q (only taken when every prime is below 2^50) for consumers that
-// multiply them in Montgomery form; otherwise canonical
+// lazy_out: outputs left below 2q (pm contexts) or 64q (others, only taken when every prime is below 2^50) for
+// consumers that multiply them in Montgomery form; otherwise canonical
 int launch_ntt_fwd(const bfhe_ctx* ctx, NttIO io, int n_polys, int n_limbs, LimbMap map, cudaStream_t st,
                    int lazy_out = 0);
 // mont != 0: the final scale is N^-1 R (undoes one Montgomery factor R^-1 of the inputs)
-// lazy_out: 0 canonical; 1 outputs below 2q (the twist product without its final subtraction) for consumers
-// that take lazy words; 2 no twist at all (words below 61q, from inputs below q) for consumers that fold the
-// twist into a product of their own (scale-and-round, mod-down)
+// lazy_out: 0 canonical; 2 no twist at all (words below 61q, or signed words below 2^63 in a pm context; from inputs
+// below q) for consumers that fold the twist into a product of their own (scale-and-round, mod-down)
 int launch_ntt_inv(const bfhe_ctx* ctx, NttIO io, int n_polys, int n_limbs, LimbMap map, int mont,
                    cudaStream_t st, int lazy_out = 0);
-int ntt_config(int logN, int inverse, int* log_m, int* log_e);
-void ntt_set_log_e(int log_e);   // tuning override (0 = default)
+int ntt_config(int logN, int inverse, size_t limbs, int* log_m, int* log_e);   // shape of a launch of `limbs` limbs

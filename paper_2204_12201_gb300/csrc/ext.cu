@@ -225,11 +225,20 @@ __device__ __forceinline__ ulonglong2 twist_at(const u64* twist, int p, int f, i
     return __ldg(reinterpret_cast<const ulonglong2*>(twist) + ((size_t)p * 3 + f) * N + k);
 }
 
+// a word times a twist entry, in [0, 2q): Shoup pairs, or pm_mul's entries when the moduli are 2^bits - d (bits > 0)
+__device__ __forceinline__ u64 twist_mul(u64 w, const ulonglong2& f, u64 q, int bits) {
+    if (bits) {
+        const uint32_t d = (uint32_t)(((u64)1 << bits) - q);
+        return pm_lazy(pm_mul(w, f, bits - 30, d << 2), q, bits, d);
+    }
+    return shoup_lazy(w, f.x, f.y, q);
+}
+
 // scale-and-round of the tensor (X slots 0..2, Q u B limbs) into C3 [n][3][L][N].  The inverse transforms
 // leave the tensor untwisted: the first product of each limb, by t, also carries the twist N^-1 psi^-k R.
 template <int NS, int KS, bool FAST>
 __global__ void __launch_bounds__(256, 2) k_scale(const u64* X, u64* C3, int n, ExtDesc eQB, ExtDesc eBQ, const u64* twist, int nP,
-                        const u64* Qinv_b, const u64* bq, int N, FastTab<FAST ? NS : 1, FAST ? KS : 1> fq,
+                        const u64* Qinv_b, const u64* bq, int N, int bits, FastTab<FAST ? NS : 1, FAST ? KS : 1> fq,
                         FastTab<FAST ? KS : 1, FAST ? NS : 1> fb) {
     const size_t total = (size_t)n * 3 * N;
     constexpr int LK = NS + KS;
@@ -245,7 +254,7 @@ __global__ void __launch_bounds__(256, 2) k_scale(const u64* X, u64* C3, int n, 
         for (int i = 0; i < NS; ++i) {
             const u64 qi = eQB.src_q[i];
             const ulonglong2 f = twist_at(twist, i, 2, k, N);
-            r[i] = shoup_lazy(d[(size_t)i * N], f.x, f.y, qi);   // [t d]_{q_i}, < 2 q_i
+            r[i] = twist_mul(d[(size_t)i * N], f, qi, bits);   // [t d]_{q_i}, < 2 q_i
         }
         // r -> B (centred), then y = (t d - r) / Q in B
         u64 y[KS];
@@ -262,7 +271,7 @@ __global__ void __launch_bounds__(256, 2) k_scale(const u64* X, u64* C3, int n, 
                 const u64 bj = bq[j];
                 const int pj = NS + (nP - 1 - NS - KS) + j;                      // prime index of b_j
                 const ulonglong2 f = twist_at(twist, pj, 2, k, N);
-                const u64 td = shoup_lazy(d[(size_t)(NS + j) * N], f.x, f.y, bj);   // [t d]_{b_j}, < 2 b_j
+                const u64 td = twist_mul(d[(size_t)(NS + j) * N], f, bj, bits);   // [t d]_{b_j}, < 2 b_j
                 u64 rb;
                 if constexpr (FAST)
                     rb = fast ? fast_eval3<NS, KS>(r0, r1, vv, eQB, fq, j) : ext_eval<NS, false>(v, neg, eQB, j);
@@ -294,7 +303,7 @@ __global__ void __launch_bounds__(256, 2) k_scale(const u64* X, u64* C3, int n, 
 // Measured at N = 32768, L = 16: mul_relin +10.6%, squarings +12.1%; at L = 8 the one-pass kernel is 1% faster.
 template <int NS, int KS>
 __global__ void __launch_bounds__(256, 2) k_scale_a(const u64* X, u64* Yt, int n, ExtDesc eQB, const u64* twist, int nP,
-                                                    const u64* Qinv_b, const u64* bq, int N, FastTab<NS, KS> fq) {
+                                                    const u64* Qinv_b, const u64* bq, int N, int bits, FastTab<NS, KS> fq) {
     const size_t total = (size_t)n * 3 * N;
     constexpr int LK = NS + KS;
     for (size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
@@ -313,7 +322,7 @@ __global__ void __launch_bounds__(256, 2) k_scale_a(const u64* X, u64* Yt, int n
 #pragma unroll
             for (int i = 0; i < NS; ++i) {
                 const ulonglong2 f = twist_at(twist, i, 2, k, N);
-                r[i] = shoup_lazy(d[(size_t)i * N], f.x, f.y, eQB.src_q[i]);
+                r[i] = twist_mul(d[(size_t)i * N], f, eQB.src_q[i], bits);
             }
             fast = fast_prep<NS, KS>(r, eQB, fq, r0, r1, vv);
         }
@@ -323,14 +332,14 @@ __global__ void __launch_bounds__(256, 2) k_scale_a(const u64* X, u64* Yt, int n
 #pragma unroll
             for (int i = 0; i < NS; ++i) {
                 const ulonglong2 f = twist_at(twist, i, 2, k, N);
-                r[i] = shoup_lazy(d[(size_t)i * N], f.x, f.y, eQB.src_q[i]);
+                r[i] = twist_mul(d[(size_t)i * N], f, eQB.src_q[i], bits);
             }
             const bool neg = garner<NS>(r, eQB, v);
             for (int j = 0; j < KS; ++j) {
                 const u64 bj = bq[j];
                 const int pj = NS + (nP - 1 - NS - KS) + j;
                 const ulonglong2 f = twist_at(twist, pj, 2, k, N);
-                const u64 td = shoup_lazy(d[(size_t)(NS + j) * N], f.x, f.y, bj);
+                const u64 td = twist_mul(d[(size_t)(NS + j) * N], f, bj, bits);
                 const u64 rb = ext_eval<NS, false>(v, neg, eQB, j);
                 yo[(size_t)j * N] = shoup_lazy(td + bj - rb, Qinv_b[j], Qinv_b[KS + j], bj);
             }
@@ -341,7 +350,7 @@ __global__ void __launch_bounds__(256, 2) k_scale_a(const u64* X, u64* Yt, int n
             const u64 bj = bq[j];
             const int pj = NS + (nP - 1 - NS - KS) + j;
             const ulonglong2 f = twist_at(twist, pj, 2, k, N);
-            const u64 td = shoup_lazy(d[(size_t)(NS + j) * N], f.x, f.y, bj);
+            const u64 td = twist_mul(d[(size_t)(NS + j) * N], f, bj, bits);
             const u64 rb = fast_eval3<NS, KS>(r0, r1, vv, eQB, fq, j);
             yo[(size_t)j * N] = shoup_lazy(td + bj - rb, Qinv_b[j], Qinv_b[KS + j], bj);
         }
@@ -379,7 +388,7 @@ __global__ void __launch_bounds__(256, 2) k_scale_b(const u64* Yt, u64* C3, int 
 // first multiplied by the twist N^-1 psi^-k R that the inverse transform left out)
 template <int NA>
 __global__ void k_moddown(const u64* W, const u64* C3, u64* out, int n, int L, ExtDesc ePQ, const u64* Pinv,
-                          const u64* qtab, const u64* twist, int N) {
+                          const u64* qtab, const u64* twist, int N, int bits) {
     // two consecutive coefficients per thread (N is even, every limb starts 16-byte aligned): 16-byte accesses
     const size_t half = (size_t)N >> 1;
     const size_t total = (size_t)n * 2 * half;
@@ -398,8 +407,8 @@ __global__ void k_moddown(const u64* W, const u64* C3, u64* out, int n, int L, E
             const ulonglong2 ww = *reinterpret_cast<const ulonglong2*>(w + (size_t)(L + a) * N);
             const ulonglong2* f = tw2 + ((size_t)(L + a) * 3 + 1) * N + k;
             const ulonglong2 f0 = __ldg(f), f1 = __ldg(f + 1);
-            x0[a] = shoup_lazy(ww.x, f0.x, f0.y, ePQ.src_q[a]);   // < 2 p_a
-            x1[a] = shoup_lazy(ww.y, f1.x, f1.y, ePQ.src_q[a]);
+            x0[a] = twist_mul(ww.x, f0, ePQ.src_q[a], bits);   // < 2 p_a
+            x1[a] = twist_mul(ww.y, f1, ePQ.src_q[a], bits);
         }
         const bool neg0 = garner<NA>(x0, ePQ, v0), neg1 = garner<NA>(x1, ePQ, v1);
         const u64* cin = C3 + (c * 3 + comp) * (size_t)L * N + k;
@@ -410,7 +419,7 @@ __global__ void k_moddown(const u64* W, const u64* C3, u64* out, int n, int L, E
             const ulonglong2 f0 = __ldg(f), f1 = __ldg(f + 1);
             const ulonglong2 ww = *reinterpret_cast<const ulonglong2*>(w + (size_t)i * N);
             const ulonglong2 cc = *reinterpret_cast<const ulonglong2*>(cin + (size_t)i * N);
-            const u64 w0 = shoup_lazy(ww.x, f0.x, f0.y, qi), w1 = shoup_lazy(ww.y, f1.x, f1.y, qi);   // < 2 q_i
+            const u64 w0 = twist_mul(ww.x, f0, qi, bits), w1 = twist_mul(ww.y, f1, qi, bits);   // < 2 q_i
             const u64 y0 = shoup(sub_mod(w0, ext_eval<NA, false>(v0, neg0, ePQ, i), qi), pw, pws, qi);
             const u64 y1 = shoup(sub_mod(w1, ext_eval<NA, false>(v1, neg1, ePQ, i), qi), pw, pws, qi);
             *reinterpret_cast<ulonglong2*>(o + (size_t)i * N) = make_ulonglong2(add_mod(cc.x, y0, qi), add_mod(cc.y, y1, qi));
@@ -522,7 +531,7 @@ __global__ void k_modup_n(const u64* A, const u64* B, u64* X, int n, int slots, 
 }
 
 __global__ void k_scale_n(const u64* X, u64* C3, int n, ExtDesc eQB, ExtDesc eBQ, const u64* twist, int nP,
-                          const u64* Qinv_b, const u64* bq, int N) {
+                          const u64* Qinv_b, const u64* bq, int N, int bits) {
     const int ns = eQB.n_src, ks = eBQ.n_src, LK = ns + ks;
     const size_t total = (size_t)n * 3 * N;
     for (size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
@@ -535,14 +544,14 @@ __global__ void k_scale_n(const u64* X, u64* C3, int n, ExtDesc eQB, ExtDesc eBQ
         u64 r[NMAX], v[NMAX], y[NMAX];
         for (int i = 0; i < ns; ++i) {
             const ulonglong2 f = twist_at(twist, i, 2, k, N);
-            r[i] = shoup_lazy(d[(size_t)i * N], f.x, f.y, eQB.src_q[i]);
+            r[i] = twist_mul(d[(size_t)i * N], f, eQB.src_q[i], bits);
         }
         const bool neg = garner_n(r, eQB, v, ns);
         for (int j = 0; j < ks; ++j) {
             const u64 bj = bq[j];
             const int pj = ns + (nP - 1 - ns - ks) + j;
             const ulonglong2 f = twist_at(twist, pj, 2, k, N);
-            const u64 td = shoup_lazy(d[(size_t)(ns + j) * N], f.x, f.y, bj);
+            const u64 td = twist_mul(d[(size_t)(ns + j) * N], f, bj, bits);
             const u64 rb = ext_eval_n(v, neg, eQB, j, ns, false);
             y[j] = shoup_lazy(td + bj - rb, Qinv_b[j], Qinv_b[ks + j], bj);
         }
@@ -605,7 +614,7 @@ int run_scale(const bfhe_ctx* ctx, const u64* X, u64* C3, int n, cudaStream_t st
     if constexpr (NS >= 10) {
         if (tmp && fast) {
             LAUNCH((k_scale_a<NS, NS + 1>), work, X, tmp, n, ctx->ext_QB, ctx->tab.twist, (int)ctx->nP,
-                   ctx->d_Qinv_b, bq, (int)ctx->N, fast_tab<NS, NS + 1>(ctx->exth_QB));
+                   ctx->d_Qinv_b, bq, (int)ctx->N, ctx->pm_bits(), fast_tab<NS, NS + 1>(ctx->exth_QB));
             LAUNCH((k_scale_b<NS, NS + 1>), work, tmp, C3, n, ctx->ext_BQ, (int)ctx->N,
                    fast_tab<NS + 1, NS>(ctx->exth_BQ));
             return BFHE_OK;
@@ -613,10 +622,11 @@ int run_scale(const bfhe_ctx* ctx, const u64* X, u64* C3, int n, cudaStream_t st
     }
     if (fast)
         LAUNCH((k_scale<NS, NS + 1, true>), work, X, C3, n, ctx->ext_QB, ctx->ext_BQ, ctx->tab.twist, (int)ctx->nP,
-               ctx->d_Qinv_b, bq, (int)ctx->N, fast_tab<NS, NS + 1>(ctx->exth_QB), fast_tab<NS + 1, NS>(ctx->exth_BQ));
+               ctx->d_Qinv_b, bq, (int)ctx->N, ctx->pm_bits(), fast_tab<NS, NS + 1>(ctx->exth_QB),
+               fast_tab<NS + 1, NS>(ctx->exth_BQ));
     else
         LAUNCH((k_scale<NS, NS + 1, false>), work, X, C3, n, ctx->ext_QB, ctx->ext_BQ, ctx->tab.twist, (int)ctx->nP,
-               ctx->d_Qinv_b, bq, (int)ctx->N, FastTab<1, 1>{}, FastTab<1, 1>{});
+               ctx->d_Qinv_b, bq, (int)ctx->N, ctx->pm_bits(), FastTab<1, 1>{}, FastTab<1, 1>{});
     return BFHE_OK;
 }
 
@@ -671,7 +681,7 @@ int launch_scale(const bfhe_ctx* ctx, const u64* X, u64* C3, int n, cudaStream_t
     SWITCH_L(ctx->L, run_scale, ctx, X, C3, n, st, tmp)
     if (ctx->L > BFHE_MAX_L) return set_error(BFHE_EINVAL, "unsupported number of data primes");
     LAUNCH(k_scale_n, (size_t)n * 3 * ctx->N, X, C3, n, ctx->ext_QB, ctx->ext_BQ, ctx->tab.twist, (int)ctx->nP,
-           ctx->d_Qinv_b, ctx->tab.q + ctx->L + ctx->alpha, (int)ctx->N);
+           ctx->d_Qinv_b, ctx->tab.q + ctx->L + ctx->alpha, (int)ctx->N, ctx->pm_bits());
     return BFHE_OK;
 }
 
@@ -684,10 +694,10 @@ int launch_moddown(const bfhe_ctx* ctx, const u64* W, const u64* C3, u64* out, i
     const size_t work = (size_t)n * ctx->N;   // two coefficients per thread
     if (ctx->alpha == 1)
         LAUNCH(k_moddown<1>, work, W, C3, out, n, (int)ctx->L, ctx->ext_PQ, ctx->d_Pinv_q, ctx->tab.q, ctx->tab.twist,
-               (int)ctx->N);
+               (int)ctx->N, ctx->pm_bits());
     else if (ctx->alpha == 2)
         LAUNCH(k_moddown<2>, work, W, C3, out, n, (int)ctx->L, ctx->ext_PQ, ctx->d_Pinv_q, ctx->tab.q, ctx->tab.twist,
-               (int)ctx->N);
+               (int)ctx->N, ctx->pm_bits());
     else
         return set_error(BFHE_EINVAL, "alpha must be 1 or 2");
     return BFHE_OK;

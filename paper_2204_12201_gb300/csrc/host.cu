@@ -8,6 +8,7 @@
 // primes, the next K the auxiliary base, K the least count with B > 2 t N Q.
 // The slot root is zeta = g^((t-1)/2N) mod t with g the least primitive root
 // of t (the encode/decode NTT uses psi = zeta, so slot j = m(zeta^(2j+1))).
+#include <algorithm>
 #include <cstdio>
 #include <cstring>
 #include <atomic>
@@ -493,6 +494,14 @@ extern "C" int bfhe_ctx_create(const bfhe_params* prm, int device, bfhe_ctx** ou
     c->nP = (uint32_t)c->primes.size();
     const uint32_t L = c->L, A = c->alpha, nP = c->nP;
 
+    // Products as pm_mul (common.cuh) when every transform stays below 2^63 in magnitude: one stage adds at most
+    // 3 2^29 4d + 2.5 2^(bits + 2); the forward starts below 4q, the inverse's first pass sums up to 32 inputs.
+    if (bits >= 45 && bits <= 55) {
+        u64 d = 0;
+        for (u64 q : rule.moduli) d = std::max(d, ((u64)1 << bits) - q);
+        const u128 g = (u128)6442450944ull * d + ((u128)5 << (bits + 1));
+        c->pm = (u128)c->logN * g + ((u128)1 << (bits + 5)) < ((u128)1 << 63);
+    }
     // bit reversal
     c->brv.resize(N);
     for (uint32_t k = 0; k < N; ++k) {
@@ -507,6 +516,7 @@ extern "C" int bfhe_ctx_create(const bfhe_params* prm, int device, bfhe_ctx** ou
     std::vector<u64> qv(c->primes), qinv(nP), mu(nP), R2(nP);
     std::vector<u64> tw((size_t)nP * N * 2), itw((size_t)nP * N * 2), twist((size_t)nP * 3 * N * 2);
     std::vector<u64> twl((size_t)nP * 3 * N * 2);
+    const bool pm_ctx = c->pm;
     for (uint32_t p = 0; p < nP; ++p) {
         const u64 q = c->primes[p];
         if (p == nP - 1 && !batching) {
@@ -522,6 +532,15 @@ extern "C" int bfhe_ctx_create(const bfhe_params* prm, int device, bfhe_ctx** ou
         R2[p] = mulmod(R, R, q);
         const u64 psi = (p == nP - 1) ? powmod(least_primitive_root(q), (q - 1) / (2 * (u64)N), q) : root_2n(q, N);
         const u64 ipsi = invmod(psi, q);
+        const bool pm = pm_ctx && p != nP - 1;
+        auto entry = [&](std::vector<u64>& t, size_t o, u64 w) {
+            if (pm) {
+                pm_entry(w, q, (int)bits, &t[o], &t[o + 1]);
+            } else {
+                t[o] = w;
+                t[o + 1] = shoup_of(w, q);
+            }
+        };
         // powers psi^k and psi^-k, k < 2N
         std::vector<u64> pw(2 * N), ipw(2 * N);
         pw[0] = ipw[0] = 1;
@@ -532,8 +551,7 @@ extern "C" int bfhe_ctx_create(const bfhe_params* prm, int device, bfhe_ctx** ou
         // forward: psi^brv(k)
         for (uint32_t k = 0; k < N; ++k) {
             const size_t o = ((size_t)p * N + k) * 2;
-            tw[o] = pw[c->brv[k]];
-            tw[o + 1] = shoup_of(tw[o], q);
+            entry(tw, o, pw[c->brv[k]]);
         }
         // the forward's last pass (E = 2^le words per thread, stages on bits b < le): the entries of stage b,
         // [N >> (b+1), N >> b), regrouped so that lanes of a warp read consecutive entries: thread tg's g-th
@@ -556,14 +574,12 @@ extern "C" int bfhe_ctx_create(const bfhe_params* prm, int device, bfhe_ctx** ou
             }
         }
         // inverse DIT: entry 2^b + j (j < 2^b) = omega^-((N >> (b+1)) j) = psi^-(2 (N >> (b+1)) j)
-        itw[(size_t)p * N * 2] = 1;
-        itw[(size_t)p * N * 2 + 1] = shoup_of(1, q);
+        entry(itw, (size_t)p * N * 2, 1);
         for (uint32_t b = 0; (1u << b) < N; ++b) {
             for (uint32_t j = 0; j < (1u << b); ++j) {
                 const size_t o = ((size_t)p * N + (1u << b) + j) * 2;
                 const u64 e = (2ull * (N >> (b + 1)) * j) % (2ull * N);
-                itw[o] = ipw[e];
-                itw[o + 1] = shoup_of(itw[o], q);
+                entry(itw, o, ipw[e]);
             }
         }
         // twist N^-1 psi^-m: plain, times R, and times t R (scale-and-round takes the multiply's inverse
@@ -574,16 +590,16 @@ extern "C" int bfhe_ctx_create(const bfhe_params* prm, int device, bfhe_ctx** ou
             const u64 vs[3] = {v0, v1, v2};
             for (int f = 0; f < 3; ++f) {
                 const size_t o = (((size_t)p * 3 + f) * N + m) * 2;
-                twist[o] = vs[f];
-                twist[o + 1] = shoup_of(vs[f], q);
+                entry(twist, o, vs[f]);
             }
         }
     }
     const size_t o_q = ar.add(qv), o_qinv = ar.add(qinv), o_mu = ar.add(mu), o_R2 = ar.add(R2);
     const size_t o_tw = ar.add(tw), o_twl = ar.add(twl), o_itw = ar.add(itw), o_twist = ar.add(twist);
     std::vector<u64> brv_packed((N + 1) / 2);
-    for (uint32_t k = 0; k < N; k += 2)
-        brv_packed[k / 2] = (u64)c->brv[k] | ((u64)(k + 1 < N ? c->brv[k + 1] : 0) << 32);
+    // slot j <-> evaluation index brv(j), stored at eval_pos of it (ntt.cu): bits 1-4 and 5-9 exchanged
+    auto eval_pos = [](uint32_t w) { return (w & ~1022u) | ((w & 30u) << 5) | ((w >> 4) & 62u); };
+    for (uint32_t k = 0; k < N; k += 2) brv_packed[k / 2] = (u64)eval_pos(c->brv[k]) | ((u64)eval_pos(c->brv[k + 1]) << 32);
     const size_t o_brv = ar.add(brv_packed);
 
     // base extensions

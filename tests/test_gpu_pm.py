@@ -1,0 +1,43 @@
+"""GPU: the multiply and the transforms on both sides of the rule that takes products modulo 2^b - d (45 to 55 bits)
+against the oracle, word for word."""
+
+import numpy as np
+import pytest
+import torch
+
+from oracle import bfv
+from oracle.params import Params
+from paper_2204_12201_gb300 import inputs
+from tests.gpu_util import assert_ct_equal, need_gpu
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("bits", [44, 45, 50, 55, 56])
+@pytest.mark.parametrize("N,L,alpha", [(1024, 3, 1), (2048, 9, 2)])
+def test_multiply_at_the_edges_of_the_product_rule(bits, N, L, alpha):
+    need_gpu()
+    import __graft_entry__
+    __graft_entry__.build()
+    from paper_2204_12201_gb300 import bfhe
+    cfg = dict(N=N, L=L, alpha=alpha, prime_bits=bits)
+    prm, ctx = Params(**cfg), bfhe.Context(**cfg)
+    ctx.keygen(5)
+    keys = bfv.keygen(prm, 5)
+    y = inputs.slots(bits, 2, N)
+    ct = ctx.encrypt(torch.from_numpy(y).cuda(), 7)
+    a, b = (bfv.encrypt(prm, keys, [int(v) for v in y[i]], 7, i) for i in range(2))
+    assert_ct_equal(prm, ct, [a, b], "encrypt")
+    prod = ctx.mul_relin(ct[:1].contiguous(), ct[1:].contiguous())
+    assert_ct_equal(prm, prod, [bfv.mul_relin(prm, keys, a, b)], "mul_relin")
+    assert np.array_equal(ctx.decrypt(ct).cpu().numpy(), y)
+    # the transform pair is the identity at the residues' extremes
+    q = torch.tensor(ctx.primes[:L], device="cuda").view(1, L, 1)
+    x = torch.randint(0, 1 << 62, (3, L, N), device="cuda") % q
+    x[0] = q[0] - 1
+    x[1] = 0
+    z = ctx.ntt(x.clone())
+    assert bool((z >= 0).all()) and bool((z < q).all())
+    assert torch.equal(ctx.ntt(z.clone(), inverse=True), x)
+    ctx.check()
+    ctx.close()
