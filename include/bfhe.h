@@ -130,7 +130,9 @@ size_t bfhe_mul_scratch_bytes(const bfhe_ctx* ctx, size_t n);
  * either way (bit for bit); only the speed differs.  Needs every modulus
  * below 2^50 and at most 16 data primes (BFHE_EINVAL otherwise).  Default: on
  * from 8 to 16 data primes (where it measured faster on GB300), off
- * otherwise.  bfhe_fast_extension
+ * otherwise.  With moduli of 45 to 55 bits and at most 16 data primes another
+ * guarded form of the same conversion runs whatever the default, unless the
+ * extension has been switched off by this call (then mixed radix alone).  bfhe_fast_extension
  * returns the current setting (1 or 0; BFHE_EINVAL for a NULL context).  The
  * paper has no counterpart: SEAL, which it runs on, uses approximate fast
  * conversions of this family. */

@@ -15,8 +15,9 @@ ROOT = os.path.dirname(PKG)
 CSRC = os.path.join(PKG, "csrc")
 LIBDIR = os.path.join(PKG, "_lib")
 OBJDIR = os.path.join(ROOT, "_build")
-# (object, source, defines): ntt.cu's kernels compile as four objects in parallel
+# (object, source, defines): the kernels of ntt.cu and ext_pm.cu compile as several objects in parallel
 UNITS = [("host", "host.cu", []), ("kernels", "kernels.cu", []), ("ext", "ext.cu", []), ("api", "api.cu", [])]
+UNITS += [("ext_pm%d" % p, "ext_pm.cu", ["-DBFHE_EXT_PM_PART=%d" % p]) for p in range(5)]
 UNITS += [("ntt%d" % p, "ntt.cu", ["-DBFHE_NTT_PART=%d" % p]) for p in range(4)]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC", "-Xcompiler", "-O2"]

@@ -64,6 +64,9 @@ int mul_relin_impl(bfhe_ctx* c, const u64* A, const u64* B, u64* out, size_t n, 
         iox.in_os = iox.out_os = 4 * LK * N;
         iox.in_is = iox.out_is = LK * N;
         iox.in_ls = iox.out_ls = N;
+        iox.src[0] = a;   // the Q limbs come straight from the inputs
+        iox.src[1] = b;
+        iox.src_limbs = (int)L;
         RC(launch_ntt_fwd(c, iox, slots * m, (int)LK, c->mapQB(), st, 1));   // tensor takes lazy words
         RC(launch_tensor(c, X, m, sq, st));
         NttIO io3;
@@ -188,6 +191,7 @@ extern "C" int bfhe_set_fast_extension(bfhe_ctx* c, int on) {
     if (on && c->L > BFHE_MAX_L_UNROLLED)
         return set_error(BFHE_EINVAL, "the fast extension is built for at most 16 data primes");
     c->fast_ext = on != 0;
+    c->exact_ext = on == 0;
     return BFHE_OK;
 }
 
@@ -736,7 +740,7 @@ int mod_to_bits_impl(bfhe_ctx* c, const u64* x, uint32_t s, u64 c_lo, u64 c_hi, 
         const u64 c_base = c_lo + cb;
         if (graph && cb > 0 && (size_t)Ct == C) {
             const std::vector<u64> key = {(u64)(uintptr_t)x, (u64)(uintptr_t)bits_out, (u64)(uintptr_t)fixed,
-                                          (u64)(uintptr_t)mul, mw, n, s, C, (u64)mode, c->fast_ext ? 1ull : 0ull};
+                                          (u64)(uintptr_t)mul, mw, n, s, C, (u64)mode, (c->fast_ext ? 1ull : 0ull) | (c->exact_ext ? 2ull : 0ull)};
             if (!c->tile_exec || c->tile_key != key)
                 RC(m2b_capture(c, key, x, s, (int)C, mode, bits_out, n, fixed, mul, mw));
             RC(launch_set_word(c->d_cbase, c_base, ws));

@@ -163,9 +163,8 @@ __device__ __forceinline__ u64 pm_canon(u64 x, u64 q, int b, uint32_t d) {
     const u64 y = pm_lazy(x, q, b, d);
     return y >= q ? y - q : y;
 }
-// host: the table entry of w
-inline void pm_entry(u64 w, u64 q, int b, u64* x, u64* y) {
-    const int k = b - 30;
+// host: the table entry of w, cut at bit k (b - 30 for pm_mul)
+inline void pm_entry(u64 w, u64 q, int k, u64* x, u64* y) {
     const u64 m = ((u64)1 << k) - 1, v = (u64)(((u128)w << 32) % q);
     *x = (w & m) | ((w >> k) << 32);
     *y = (v & m) | ((v >> k) << 32);
@@ -209,6 +208,16 @@ struct ExtHost {
     std::vector<u64> qhinv, qhinv_s, g_hi, g_lo;     // [n]
 };
 
+// Host constants of an extension sum for moduli 2^b - d (ext_pm.cu): words cut at bit k = b - 28
+struct PmSum {
+    int n = 0, m = 0;
+    std::vector<uint32_t> c;          // [m][n][4] (l, h) of the constant and of 2^hs times it, hs = (b + 2) / 2
+    std::vector<uint32_t> cv, d;      // [m][2] the overflow count's constant, [m] d of the target
+    std::vector<uint32_t> w, dsrc;    // [n][4] (S/s_i)^-1 in the same form, [n] d of the source
+    std::vector<u64> q;               // [n]
+    u64 guard = 0;                    // bound of 2^b |sum y_i / s_i - sum y_i / 2^b|
+};
+
 // Device-side prime tables of a context, by prime index
 // (0..L-1 data, L..L+alpha-1 special, L+alpha..L+alpha+K-1 auxiliary, last: t).  The pairs of tw, twl, itw and
 // twist are pm_mul's entries for the moduli of a context with pm set, (w, Shoup(w)) otherwise and always for t.
@@ -244,6 +253,10 @@ struct bfhe_ctx {
     uint32_t* d_brv = nullptr;   // [N] storage position of slot j's evaluation
     ExtDesc ext_QB{}, ext_BQ{}, ext_PQ{}, ext_Qt{};
     ExtHost exth_QB, exth_BQ;
+    // pm contexts of at most 16 data primes: the input extension, scale-and-round's two sums and its twist table
+    // [L + K][N] (data: t R N^-1 psi^-k (Q/q_i)^-1; auxiliary: t R N^-1 psi^-k Q^-1 (B/b_j)^-1; words cut at b - 28)
+    PmSum pm_up, pm_toB, pm_toQ;
+    const ulonglong2* d_xtw = nullptr;
     // Shoup pair tables: p[i] = w_i, p[n + i] = ws_i
     const u64* d_tmod = nullptr;    // [nP] [t]_{prime}
     const u64* d_delta_q = nullptr; // [L]  [Delta]_{q_i}
@@ -272,6 +285,9 @@ struct bfhe_ctx {
 
     uint64_t counts[4] = {0, 0, 0, 0};
     bool fast_ext = false;       // guarded fast base extension in the multiply (bfhe_set_fast_extension)
+    bool exact_ext = false;      // the caller has switched it off: mixed radix everywhere
+    bool pm_ext = false;         // the extensions of ext_pm.cu are available (at most 16 primes, pm)
+    bool use_pm_ext() const { return pm_ext && !exact_ext; }
 
     // mod_to_bits tiles replayed from a CUDA graph (bfhe_set_graph_tiles): the tile is captured once on a
     // context-owned stream and replayed with its candidate base in the device word d_cbase; the
@@ -352,6 +368,10 @@ struct NttIO {
     size_t in_os, in_is, in_ls;
     size_t out_os, out_is, out_ls;
     bool natural = false;   // the evaluation side in bit-reversed index order (bfhe_ntt) rather than the storage order
+    // forward only: limbs below src_limbs of poly (outer, inner) are read from src[inner >> 1], ciphertexts
+    // [outer][2][src_limbs][N] of which inner & 1 selects the polynomial (the multiply's inputs, which need no copy)
+    const u64* src[2] = {nullptr, nullptr};
+    int src_limbs = 0;
 };
 // contiguous [n_polys][n_limbs][N] in and out
 inline NttIO ntt_io(const u64* in, u64* out, size_t n_limbs, size_t N) {

@@ -230,6 +230,43 @@ ExtOffsets build_ext(Arena& ar, const std::vector<u64>& src, const std::vector<u
     return o;
 }
 
+// Constants of sum_i y_i c_ij + v cv_j over the targets dst (ext_pm.cu); ymax bounds the digits y_i
+PmSum pm_sum(const std::vector<u64>& src, const std::vector<u64>& dst, int b, u128 ymax,
+             const std::vector<std::vector<u64>>& c, const std::vector<u64>& cv) {
+    PmSum s;
+    s.n = (int)src.size();
+    s.m = (int)dst.size();
+    const int k = b - 28, hs = (b + 2) / 2;
+    const u64 mask = ((u64)1 << k) - 1;
+    auto put = [&](std::vector<uint32_t>& o, u64 w) {
+        o.push_back((uint32_t)(w & mask));
+        o.push_back((uint32_t)(w >> k));
+    };
+    u64 dmax = 0;
+    for (int i = 0; i < s.n; ++i) {
+        const u64 q = src[i];
+        u64 h = 1;
+        for (int m = 0; m < s.n; ++m)
+            if (m != i) h = mulmod(h, src[m] % q, q);
+        const u64 w = invmod(h, q);   // (S/s_i)^-1
+        put(s.w, w);
+        put(s.w, (u64)(((u128)w << hs) % q));
+        s.q.push_back(q);
+        s.dsrc.push_back((uint32_t)(((u64)1 << b) - q));
+        dmax = std::max(dmax, ((u64)1 << b) - q);
+    }
+    for (int j = 0; j < s.m; ++j) {
+        for (int i = 0; i < s.n; ++i) {
+            put(s.c, c[j][i]);
+            put(s.c, (u64)(((u128)c[j][i] << hs) % dst[j]));
+        }
+        put(s.cv, cv[j]);
+        s.d.push_back((uint32_t)(((u64)1 << b) - dst[j]));
+    }
+    s.guard = (u64)((u128)s.n * ymax * dmax / (((u64)1 << b) - dmax)) + s.n + 2;
+    return s;
+}
+
 ExtDesc ext_ptrs(const u64* base, const ExtOffsets& o) {
     ExtDesc d;
     d.n_src = o.n;
@@ -495,12 +532,13 @@ extern "C" int bfhe_ctx_create(const bfhe_params* prm, int device, bfhe_ctx** ou
     const uint32_t L = c->L, A = c->alpha, nP = c->nP;
 
     // Products as pm_mul (common.cuh) when every transform stays below 2^63 in magnitude: one stage adds at most
-    // 3 2^29 4d + 2.5 2^(bits + 2); the forward starts below 4q, the inverse's first pass sums up to 32 inputs.
+    // 3 2^29 4d + 2.5 2^(bits + 2); the forward starts below 2^60 (the lift's sums, 2^(bits + 1) above 52 bits), the
+    // inverse's first pass sums up to 32 inputs.
     if (bits >= 45 && bits <= 55) {
         u64 d = 0;
         for (u64 q : rule.moduli) d = std::max(d, ((u64)1 << bits) - q);
         const u128 g = (u128)6442450944ull * d + ((u128)5 << (bits + 1));
-        c->pm = (u128)c->logN * g + ((u128)1 << (bits + 5)) < ((u128)1 << 63);
+        c->pm = (u128)c->logN * g + ((u128)1 << (bits > 52 ? bits + 5 : 60)) < ((u128)1 << 63);
     }
     // bit reversal
     c->brv.resize(N);
@@ -535,7 +573,7 @@ extern "C" int bfhe_ctx_create(const bfhe_params* prm, int device, bfhe_ctx** ou
         const bool pm = pm_ctx && p != nP - 1;
         auto entry = [&](std::vector<u64>& t, size_t o, u64 w) {
             if (pm) {
-                pm_entry(w, q, (int)bits, &t[o], &t[o + 1]);
+                pm_entry(w, q, (int)bits - 30, &t[o], &t[o + 1]);
             } else {
                 t[o] = w;
                 t[o + 1] = shoup_of(w, q);
@@ -610,6 +648,60 @@ extern "C" int bfhe_ctx_create(const bfhe_params* prm, int device, bfhe_ctx** ou
     const ExtOffsets eQB = build_ext(ar, Qp, Bp, &c->exth_QB), eBQ = build_ext(ar, Bp, Qp, &c->exth_BQ),
                      ePQ = build_ext(ar, Pp, Qp), eQt = build_ext(ar, Qp, Tp);
 
+    // the same extensions for moduli 2^b - d
+    size_t o_xtw = 0;
+    const bool pm_ext = c->pm && L <= BFHE_MAX_L_UNROLLED;
+    if (pm_ext) {
+        const int b = (int)bits, hs = (b + 2) / 2;
+        auto part = [](const std::vector<u64>& s, int skip, u64 m) {   // product of s without s[skip], mod m
+            u64 r = 1 % m;
+            for (int i = 0; i < (int)s.size(); ++i)
+                if (i != skip) r = mulmod(r, s[i] % m, m);
+            return r;
+        };
+        u64 d = 0;
+        for (uint32_t p = 0; p + 1 < nP; ++p) d = std::max(d, ((u64)1 << bits) - c->primes[p]);
+        // digits of the inputs' extension, and of scale-and-round's (folded once)
+        const u128 y_up = ((u128)1 << b) + ((u128)d << (hs + 1)) + ((u128)1 << (hs + b - 27));
+        const u128 y_sc = ((u128)1 << b) + ((u128)d << (63 - b));
+        std::vector<std::vector<u64>> up(K, std::vector<u64>(L)), toB(K, std::vector<u64>(L)), toQ(L, std::vector<u64>(K));
+        std::vector<u64> v_up(K), v_toB(K), v_toQ(L), bh(K), fold(L + K);
+        for (int j = 0; j < K; ++j) {
+            const u64 m = Bp[j], Qm = part(Qp, -1, m);
+            bh[j] = invmod(part(Bp, j, m), m);
+            for (uint32_t i = 0; i < L; ++i) {
+                up[j][i] = part(Qp, (int)i, m);
+                toB[j][i] = mulmod(m - invmod(Qp[i] % m, m), bh[j], m);   // -(1/q_i) (B/b_j)^-1
+            }
+            v_up[j] = (m - Qm) % m;
+            v_toB[j] = bh[j];
+            fold[L + j] = mulmod(invmod(Qm, m), bh[j], m);
+        }
+        for (uint32_t i = 0; i < L; ++i) {
+            const u64 m = Qp[i];
+            for (int j = 0; j < K; ++j) toQ[i][j] = part(Bp, j, m);
+            v_toQ[i] = (m - part(Bp, -1, m)) % m;
+            fold[i] = invmod(part(Qp, (int)i, m), m);
+        }
+        c->pm_up = pm_sum(Qp, Bp, b, y_up, up, v_up);
+        c->pm_toB = pm_sum(Qp, Bp, b, y_sc, toB, v_toB);
+        c->pm_toQ = pm_sum(Bp, Qp, b, y_sc, toQ, v_toQ);
+        // twist rows: t R N^-1 psi^-k of row 2 times the folded constant
+        std::vector<u64> xtw((size_t)(L + K) * N * 2);
+        for (uint32_t l = 0; l < L + K; ++l) {
+            const uint32_t p = l < L ? l : l + A;
+            const u64 q = c->primes[p];
+            for (uint32_t m = 0; m < N; ++m) {
+                const size_t o = (((size_t)p * 3 + 2) * N + m) * 2;
+                const u64 mask = ((u64)1 << (bits - 30)) - 1;
+                const u64 w = (twist[o] & mask) | ((twist[o] >> 32) << (bits - 30));   // the entry's constant
+                const size_t x = ((size_t)l * N + m) * 2;
+                pm_entry(mulmod(w, fold[l], q), q, b - 28, &xtw[x], &xtw[x + 1]);
+            }
+        }
+        o_xtw = ar.add(xtw);
+    }
+
     // scalar constants
     u64 Qt = 1;
     for (u64 q : Qp) Qt = mulmod(Qt, q % t, t);
@@ -670,7 +762,11 @@ extern "C" int bfhe_ctx_create(const bfhe_params* prm, int device, bfhe_ctx** ou
     c->ext_BQ = ext_ptrs(base, eBQ);
     c->ext_PQ = ext_ptrs(base, ePQ);
     c->ext_Qt = ext_ptrs(base, eQt);
-    // the guarded fast extension measures faster from 8 data primes up (slower at 2)
+    if (pm_ext) c->d_xtw = reinterpret_cast<const ulonglong2*>(base + o_xtw);
+    // the guarded fast extension of ext.cu measures faster from 8 data primes up (slower at 2); that of ext_pm.cu, for
+    // moduli 2^b - d, at every size (64 pairs, lift + scale-and-round: N = 4096, L = 2: 61 -> 43 us, N = 8192, L = 4:
+    // 242 -> 138), so it also replaces the mixed-radix path where the setting is off by default
+    c->pm_ext = pm_ext;
     c->fast_ext = c->L >= 8 && c->L <= BFHE_MAX_L_UNROLLED && c->ext_QB.fast_ok && c->ext_BQ.fast_ok;
     c->d_tmod = base + o_tmod;
     c->d_delta_q = base + o_delta;

@@ -57,6 +57,8 @@ struct NttArgs {
     u64* out;
     int n_inner;
     size_t in_os, in_is, in_ls, out_os, out_is, out_ls;
+    const u64 *src0, *src1;   // limbs below src_limbs come from here (NttIO::src)
+    int src_limbs;
     int n_limbs;
     LimbMap map;
     PrimeTab tab;
@@ -95,18 +97,30 @@ __device__ __forceinline__ int eval_pos(int w) {
     return (w & ~1022) | ((w & 30) << 5) | ((w >> 4) & 62);
 }
 
+// a 16-byte load that the compiler issues where it stands: all of a thread's first-pass words are then in flight
+// before its first butterfly (left to itself it sinks half of them between the butterflies, which a thread of the
+// inverse's first pass, mostly additions, then waits for: 511 -> 479 us for 4352 limbs at N = 16384)
+__device__ __forceinline__ ulonglong2 load_now(const ulonglong2* p) {
+    ulonglong2 v;
+    asm volatile("ld.global.v2.u64 {%0, %1}, [%2];" : "=l"(v.x), "=l"(v.y) : "l"(p));
+    return v;
+}
+
 struct LimbPtrs {
     const u64* in;   // limb start
     u64* out;        // limb start
     int p;
 };
 
+template <bool FWD>
 __device__ __forceinline__ LimbPtrs limb_ptrs(const NttArgs& a, int bx) {
     const int limb = bx % a.n_limbs;
     const int poly = bx / a.n_limbs;
     const int outer = poly / a.n_inner, inner = poly % a.n_inner;
     LimbPtrs r;
-    r.in = a.in + outer * a.in_os + inner * a.in_is + limb * a.in_ls;
+    r.in = FWD && limb < a.src_limbs
+               ? (inner < 2 ? a.src0 : a.src1) + ((size_t)(2 * outer + (inner & 1)) * a.src_limbs + limb) * a.N
+               : a.in + outer * a.in_os + inner * a.in_is + limb * a.in_ls;
     r.out = a.out + outer * a.out_os + inner * a.out_is + limb * a.out_ls;
     r.p = a.map(limb);
     return r;
@@ -201,6 +215,8 @@ __device__ __forceinline__ void fwd_pass(u64 (&x)[1 << LOG_E], u64* sm, int tid,
 #pragma unroll
         for (int e = 0; e < E; ++e) x[e] = sm[pb + poff<W_LO>(e)];
     }
+    // the compiler does not move the first butterflies up between the loads (516 -> 504 us for 4352 limbs, N = 16384)
+    if (P == 0 && !TOP) __syncwarp();
     constexpr int LOG_N = TOP ? LOG_M + 1 : LOG_M;
     // thread index over the whole limb (last pass): (jglob - N + base) / E
     const ulonglong2* twc = W_LO == 0 ? twl + ((((u64)half << LOG_M) + base) >> LOG_E) : twl;
@@ -219,7 +235,7 @@ __device__ __forceinline__ void fwd_pass(u64 (&x)[1 << LOG_E], u64* sm, int tid,
             if constexpr (PM) x[e] = LAZY ? pm_lazy(x[e], m.q, m.b, m.d) : pm_canon(x[e], m.q, m.b, m.d);
             else if constexpr (!LAZY) x[e] = reduce64(x[e], m.q, mu);
         }
-        if (natural) {
+        if (!LAZY && natural) {   // bfhe_ntt
             ulonglong2* o2 = reinterpret_cast<ulonglong2*>(out + base);
 #pragma unroll
             for (int e = 0; e < E / 2; ++e) o2[e] = make_ulonglong2(x[2 * e], x[2 * e + 1]);
@@ -234,7 +250,7 @@ __device__ __forceinline__ void fwd_pass(u64 (&x)[1 << LOG_E], u64* sm, int tid,
 template <bool PM, int LOG_M, int LOG_E, bool TOP, bool LAZY>
 __global__ void __launch_bounds__(1 << (LOG_M - LOG_E), (LOG_M < 14 && LOG_M - LOG_E <= 8 ? 2 : 1)) k_ntt_fwd(NttArgs a) {
     extern __shared__ u64 sm[];
-    const LimbPtrs lp = limb_ptrs(a, blockIdx.x);
+    const LimbPtrs lp = limb_ptrs<true>(a, blockIdx.x);
     const int half = blockIdx.y;
     const Mod<PM> m(a.tab.q[lp.p], a.bits);
     const u64 mu = PM ? 0 : a.tab.mu[lp.p];
@@ -303,11 +319,11 @@ __device__ __forceinline__ void inv_pass(u64 (&x)[1 << LOG_E], u64* sm, int tid,
     const int pb = phys(base);
     if (P == 0) {
         // W_LO == 0: E consecutive words per thread
-        if (natural) {
+        if (OUT == 0 && natural) {   // bfhe_ntt
             const ulonglong2* i2 = reinterpret_cast<const ulonglong2*>(in + base);
 #pragma unroll
             for (int e = 0; e < E / 2; ++e) {
-                const ulonglong2 v = i2[e];
+                const ulonglong2 v = load_now(i2 + e);
                 x[2 * e] = v.x;
                 x[2 * e + 1] = v.y;
             }
@@ -315,7 +331,7 @@ __device__ __forceinline__ void inv_pass(u64 (&x)[1 << LOG_E], u64* sm, int tid,
             const ulonglong2* i2 = reinterpret_cast<const ulonglong2*>(in + eval_pos(base));
 #pragma unroll
             for (int e = 0; e < E / 2; ++e) {
-                const ulonglong2 v = i2[e * 32];
+                const ulonglong2 v = load_now(i2 + e * 32);
                 x[2 * e] = v.x;
                 x[2 * e + 1] = v.y;
             }
@@ -384,7 +400,7 @@ __device__ __forceinline__ void inv_pass(u64 (&x)[1 << LOG_E], u64* sm, int tid,
 template <bool PM, int LOG_M, int LOG_E, int MODE, int OUT>
 __global__ void __launch_bounds__(1 << (LOG_M - LOG_E), (MODE == 2 && LOG_M < 14 && LOG_M - LOG_E <= 8 ? 2 : 1)) k_ntt_inv(NttArgs a) {
     extern __shared__ u64 sm[];
-    const LimbPtrs lp = limb_ptrs(a, blockIdx.x);
+    const LimbPtrs lp = limb_ptrs<false>(a, blockIdx.x);
     const int half = blockIdx.y;
     const Mod<PM> m(a.tab.q[lp.p], a.bits);
     const ulonglong2* itw = reinterpret_cast<const ulonglong2*>(a.tab.itw) + (size_t)lp.p * a.N;
@@ -545,6 +561,9 @@ NttArgs make_args(const bfhe_ctx* ctx, const NttIO& io, int n_limbs, LimbMap map
     a.tab = ctx->tab;
     a.N = (int)ctx->N;
     a.logN = (int)ctx->logN;
+    a.src0 = io.src[0];
+    a.src1 = io.src[1];
+    a.src_limbs = io.src_limbs;
     a.natural = io.natural;
     a.bits = (int)ctx->prime_bits;
     a.mont = mont;
@@ -561,21 +580,19 @@ int env_int(const char* name) {
 }  // namespace
 
 // Block size and registers per thread.  Defaults (measured on GB300 inside the multiply, pm products, us per
-// launch class): N <= 4096 in one block of 16 words per thread (64 pairs at N = 4096, L = 2: forward 55, inverse 43;
-// 32 words 61 / 88, halves 57 / 55).  N = 8192 in one block, forward at 32 words (64 pairs, L = 4: 211 against 239 at
-// 16), inverse at 16 (149 against 151).  N = 16384 forward in one block, inverse as two 8192-word halves, 32 words
-// each (64 pairs, L = 8: 1100 and 523; halves / one block 1120 / 525).  N = 32768 as two 16384-word halves, 32 words
-// (8 pairs, L = 16: 951 and 322; 16 words 974 / 477).  A launch at N = 16384 whose halves fit the 152 SMs at
-// one CTA each takes halves at 16 words, twice the threads on each limb (one pair, L = 8: 33 and 33 against 45 and
-// 42).  bfhe_ntt_config (the autotuner) or BFHE_NTT_LOG_M / BFHE_NTT_LOG_E override the defaults.
+// launch class, forward / inverse): N <= 4096 in one block of 16 words per thread (64 pairs at N = 4096, L = 2: 52 / 41;
+// 32 words 59 / 88, halves 54 / 53).  N = 8192 in one block of 32 words (64 pairs, L = 4: 201 / 147; 16 words 231 /
+// 152).  N = 16384 in one block of 32 words (64 pairs, L = 8: 1022 / 516; halves 1031 / 560).  N = 32768 as two
+// 16384-word halves, 32 words (8 pairs, L = 16: 889 / 348; 16 words 950 / 475).  A launch at N = 16384 whose halves
+// fit the 152 SMs at one CTA each takes halves at 16 words, twice the threads on each limb (one pair, L = 8: 33 / 33
+// against 44 / 42).  bfhe_ntt_config (the autotuner) or BFHE_NTT_LOG_M / BFHE_NTT_LOG_E override the defaults.
 int g_cfg[16][2][2] = {};   // [logN][inverse] -> (log_m, log_e), 0 = default
 
 int ntt_config(int logN, int inverse, size_t limbs, int* log_m, int* log_e) {
     static const int env_m = env_int("BFHE_NTT_LOG_M");
     static const int env_e = env_int("BFHE_NTT_LOG_E");
     int m = logN <= 14 ? logN : logN - 1;
-    if (inverse && logN == 14) m = 13;
-    int e = (logN >= 14 || (logN == 13 && !inverse)) ? 5 : 4;
+    int e = logN >= 13 ? 5 : 4;
     if (logN == 14 && 2 * limbs <= 152) {
         m = 13;
         e = 4;

@@ -41,3 +41,32 @@ def test_multiply_at_the_edges_of_the_product_rule(bits, N, L, alpha):
     assert torch.equal(ctx.ntt(z.clone(), inverse=True), x)
     ctx.check()
     ctx.close()
+
+
+@pytest.mark.parametrize("bits", [45, 50, 55])
+@pytest.mark.parametrize("L,alpha", [(1, 1), (2, 1), (7, 2), (8, 1), (9, 1), (12, 1), (13, 1), (15, 2), (16, 1)])
+def test_extension_forms_agree(bits, L, alpha):
+    """The multiply with the extensions for moduli 2^b - d (the default) and with mixed radix alone, on uniform
+    residues with every eighth coefficient at, or one off, the centring boundary, zero or the largest integer."""
+    need_gpu()
+    import __graft_entry__
+    __graft_entry__.build()
+    from paper_2204_12201_gb300 import bfhe
+    N = 1024
+    ctx = bfhe.Context(N=N, L=L, alpha=alpha, prime_bits=bits)
+    ctx.keygen(9)
+    Q = 1
+    for p in ctx.primes[:L]:
+        Q *= p
+    g = torch.Generator(device="cuda").manual_seed(L)
+    q = torch.tensor(ctx.primes[:L], device="cuda").view(1, 1, L, 1)
+    a, b = (torch.randint(0, 1 << 62, (3, 2, L, N), device="cuda", generator=g) % q for _ in range(2))
+    for t, x in enumerate([Q // 2, Q // 2 + 1, 0, 1, Q - 1, Q // 2 - 1]):
+        a[0, :, :, t::8] = torch.tensor([x % p for p in ctx.primes[:L]], device="cuda").view(1, L, 1)
+    new = [ctx.mul_relin(a, b), ctx.mul_relin(a, a)]
+    assert ctx.lib.bfhe_set_fast_extension(ctx.h, 0) == 0
+    old = [ctx.mul_relin(a, b), ctx.mul_relin(a, a)]
+    for x, y in zip(new, old):
+        assert torch.equal(x, y)
+    ctx.check()
+    ctx.close()

@@ -73,6 +73,102 @@ def test_products_are_congruent_and_bounded(bits, N, L):
                 assert (T - a * w) % q == 0 and abs(T) <= stage_bound(bits, d)
 
 
+class Sum:
+    """One extension sum as ext_pm.cu computes it: digits y cut at bit hs, constants at bit k, wide sums P and Q."""
+
+    def __init__(self, b):
+        self.b, self.k, self.hs = b, b - 28, (b + 2) // 2
+
+    def digits(self, ys):
+        out = []
+        for y in ys:
+            y0, y1 = u32(y & ((1 << self.hs) - 1)), s32(y >> self.hs)
+            out.append((y0, y1))
+        return out
+
+    def fold(self, ys, v, consts, cv, T, extra=None):
+        """sum y c + v cv (+ a 64-bit word times a twist constant): congruent, every partial sum below 2^63."""
+        m, P, Q = (1 << self.k) - 1, 0, 0
+
+        def acc(a, c):
+            nonlocal P, Q
+            P += a * s32(c & m)
+            Q += a * s32(c >> self.k)
+            assert abs(P) < 1 << 63 and abs(Q) < 1 << 63
+        if extra:
+            a, w = extra
+            acc(u32(a & 0xFFFFFFFF), w)
+            acc(s32(a >> 32), (w << 32) % T)
+        acc(v, cv)
+        for (y0, y1), c in zip(self.digits(ys), consts):
+            acc(y0, c)
+            acc(y1, (c << self.hs) % T)
+        d16 = s32(16 * ((1 << self.b) - T))
+        r = P + ((Q & 0xFFFFFFFF) << self.k) + s32(Q >> 32) * d16
+        assert abs(r) < 1 << 62
+        return r
+
+    def round(self, ys, guard):
+        z = sum(ys) + (1 << (self.b - 1))
+        frac = z & ((1 << self.b) - 1)
+        return z >> self.b, guard <= frac < (1 << self.b) - guard
+
+
+@pytest.mark.parametrize("bits", [45, 50, 55])
+@pytest.mark.parametrize("N,L", [(1024, 1), (16384, 8), (32768, 16)])
+def test_extension_sums_are_exact(bits, N, L):
+    """The lift's digits, overflow count and sums, and scale-and-round's with its twist word, at the extremes of their
+    operands and near the centring boundary: the guarded count is the true one and the result congruent."""
+    from fractions import Fraction
+    prm = Params(N=N, L=L, alpha=2, prime_bits=bits)
+    S, rng = Sum(bits), random.Random(bits + N)
+    src, dst = prm.q, prm.b
+    Q = 1
+    for q in src:
+        Q *= q
+    dmax = max((1 << bits) - q for q in prm.q + prm.p + prm.b)
+    hat = [pow(Q // q, -1, q) for q in src]
+    y_up = (1 << bits) + (dmax << (S.hs + 1)) + (1 << (S.hs + bits - 27))
+    y_sc = (1 << bits) + (dmax << (63 - bits))
+
+    def guard(y):
+        ds = max((1 << bits) - q for q in src)
+        return len(src) * y * ds // ((1 << bits) - ds) + len(src) + 2
+    xs = [0, 1, Q - 1, Q // 2, Q // 2 + 1, Q // 2 + Q // (1 << 40)] + [rng.randrange(Q) for _ in range(6)]
+    hit = 0
+    for x in xs:
+        ys = []
+        for q, h in zip(src, hat):
+            r, d = x % q, (1 << bits) - q
+            x0, x1 = u32(r & ((1 << S.hs) - 1)), u32(r >> S.hs)
+            hv = (h << S.hs) % q
+            q2 = x0 * (h >> S.k) + x1 * (hv >> S.k)
+            m = (1 << S.k) - 1
+            y = ((q2 & ((1 << 28) - 1)) << S.k) + x0 * (h & m) + x1 * (hv & m) + u32(q2 >> 28) * d
+            assert 0 <= y <= y_up and (y - r * h) % q == 0
+            ys.append(y)
+        v, ok = S.round(ys, guard(y_up))
+        true_v = (sum(Fraction(y, q) for y, q in zip(ys, src)) + Fraction(1, 2)).__floor__()
+        centred = x if x <= Q // 2 else x - Q
+        if ok:
+            assert v == true_v
+            hit += 1
+            for T in dst[:3] + dst[-1:]:
+                got = S.fold(ys, v, [(Q // q) % T for q in src], -Q % T, T)
+                assert bits > 52 or 0 <= got < 1 << 60   # what the forward transform's bound starts from
+                assert (got - centred) % T == 0
+    assert hit >= 8
+    # scale-and-round's first sum: folded digits (signed) and a full signed tensor word
+    for T in dst[:2]:
+        for lim in (0, 1):
+            ys = [(y_sc - 1) if lim else -(dmax << (63 - bits)) for _ in src]
+            for a in ((1 << 63) - 1, -(1 << 63), 0):
+                cs, cv, w = [T - 1] * len(src), T - 1, T - 1
+                v = S.round(ys, guard(y_sc))[0]
+                got = S.fold(ys, v, cs, cv, T, (a, w))
+                assert (got - (sum(y * c for y, c in zip(ys, cs)) + v * cv + a * w)) % T == 0
+
+
 def eval_pos(w):
     return (w & ~1022) | ((w & 30) << 5) | ((w >> 4) & 62)
 
