@@ -568,7 +568,7 @@ extern "C" int bfhe_gate_level(bfhe_ctx* c, uint64_t* wires, size_t n_wires, siz
         RC(scratch_for(c, 3 * n_mul * ctw, n_mul * n, &fixed, &mul, &mw));
         u64* AB = fixed;
         u64* P = fixed + 2 * n_mul * ctw;
-        RC(launch_gather(c, AB, wires, n, table, (int)n_mul, 0, 0, st));
+        RC(launch_gather(c, AB, wires, n, table, (int)n_mul, st));
         RC(mul_relin_impl(c, AB, AB + n_mul * ctw, P, n_mul * n, mul, mw, st));
         RC(launch_gate_epilogue(c, wires, n, table, (int)n_gates, P, (int)n_mul, st));
         c->counts[2] += n_mul * n;

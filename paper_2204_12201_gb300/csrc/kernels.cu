@@ -314,28 +314,6 @@ __global__ void k_permute(const u64* in, u64* out, const uint32_t* brv, int n, i
     }
 }
 
-__global__ void k_enc_finish(u64* ct, const u64* M, const i64* e1, const i64* e2, int n, int L, const u64* qtab,
-                             const u64* delta, int N, u64 t, uint32_t* flags) {
-    const size_t total = (size_t)n * L * N;
-    for (size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
-         idx += (size_t)gridDim.x * blockDim.x) {
-        const int k = (int)(idx % N);
-        const int i = (int)((idx / N) % L);
-        const size_t c = idx / ((size_t)N * L);
-        const u64 q = qtab[i];
-        const u64 m = M[c * N + k];
-        if (i == 0 && m >= t) atomicOr(flags, BFHE_FLAG_PLAINTEXT);   // plaintext coefficients must be < t
-        const i64 a = e1[c * N + k], b = e2[c * N + k];
-        u64* c0 = ct + (c * 2 * L + i) * N + k;
-        u64* c1 = c0 + (size_t)L * N;
-        u64 v = add_mod(*c0, shoup(m, delta[i], delta[L + i], q), q);
-        v = a >= 0 ? add_mod(v, (u64)a, q) : sub_mod(v, (u64)(-a), q);
-        *c0 = v;
-        u64 w = *c1;
-        *c1 = b >= 0 ? add_mod(w, (u64)b, q) : sub_mod(w, (u64)(-b), q);
-    }
-}
-
 // out = -(as + e) [+ [P]_{q_j} s2 on limb j of poly j when gadget]
 __global__ void k_neg_add_small(const u64* as, const i64* e, u64* out, int n_polys, int n_limbs, LimbMap map,
                                 PrimeTab tab, const u64* s2, int gadget, const u64* Pq, int L, int N) {
@@ -381,113 +359,189 @@ __constant__ int c_gate_coef[8][5] = {
     {0, 0, 0, 1, 1},     // MUX  = x (y - z) + z
 };
 
-__device__ __forceinline__ u64 lin_word(int cc, int cx, int cy, int cz, int cp, u64 cval, const u64* x,
-                                        const u64* y, const u64* z, const u64* p, size_t o, int comp, int k,
-                                        u64 q, u64 dw, u64 dws) {
-    u64 acc = 0;
-    if (cc != 0 && comp == 0 && k == 0) acc = apply(acc, shoup(cval, dw, dws, q), cc, q);
-    if (cx) acc = apply(acc, x[o], cx, q);
-    if (cy) acc = apply(acc, y[o], cy, q);
-    if (cz) acc = apply(acc, z[o], cz, q);
-    if (cp) acc = apply(acc, p[o], cp, q);
+// ---- rows: a kernel over whole limbs.  A block of 256 threads takes 256 W consecutive words of one limb (row), W = 2 as
+// one 16-byte access per thread, W = 1 where a caller's buffer is only 8-byte aligned, so that the limb, its modulus
+// and everything that hangs on them are computed once per block and not by divisions per word (bound: HBM; the genotype
+// dot product's additions of 48 ciphertexts at N = 16384, L = 8: 86 -> 47 us, 6.5 TB/s; a level of 31 gates at N = 8192,
+// L = 4: gather 16 -> 10, epilogue 17 -> 9 us).
+template <int W>
+struct Words {
+    u64 v[W];
+};
+template <int W>
+__device__ __forceinline__ Words<W> load_words(const u64* p) {
+    Words<W> r;
+    if constexpr (W == 2) {
+        const ulonglong2 t = *reinterpret_cast<const ulonglong2*>(p);
+        r.v[0] = t.x;
+        r.v[1] = t.y;
+    } else {
+        r.v[0] = *p;
+    }
+    return r;
+}
+template <int W>
+__device__ __forceinline__ void store_words(u64* p, const Words<W>& r) {
+    if constexpr (W == 2) *reinterpret_cast<ulonglong2*>(p) = make_ulonglong2(r.v[0], r.v[1]);
+    else *p = r.v[0];
+}
+// row of this block and the thread's first word in it
+template <int W>
+struct Row {
+    uint32_t row;
+    int k;
+    size_t off;   // row N + k
+    __device__ __forceinline__ explicit Row(int logN) {
+        const int sh = logN - (W == 2 ? 9 : 8);   // N >= 1024
+        row = blockIdx.x >> sh;
+        k = (int)(((blockIdx.x & ((1u << sh) - 1u)) * TPB + threadIdx.x) * W);
+        off = ((size_t)row << logN) + k;
+    }
+};
+inline bool aligned16(const void* p) { return ((uintptr_t)p & 15) == 0; }
+
+// linear combinations, W words (coefficient k onwards of limb i; the constant sits at coefficient 0 of c0)
+template <int W>
+__device__ __forceinline__ Words<W> lin_words(int cc, int cx, int cy, int cz, int cp, u64 cval, const u64* x, const u64* y,
+                                              const u64* z, const u64* p, size_t o, bool first, u64 q, u64 dw, u64 dws) {
+    Words<W> acc{};
+    if (cc != 0 && first) acc.v[0] = apply(0, shoup(cval, dw, dws, q), cc, q);
+    auto term = [&](const u64* s, int c) {
+        const Words<W> t = load_words<W>(s + o);
+#pragma unroll
+        for (int w = 0; w < W; ++w) acc.v[w] = apply(acc.v[w], t.v[w], c, q);
+    };
+    if (cx) term(x, cx);
+    if (cy) term(y, cy);
+    if (cz) term(z, cz);
+    if (cp) term(p, cp);
     return acc;
 }
 
-__global__ void k_lincomb(u64* out, const u64* x, const u64* y, const u64* z, const u64* p, LinCoef cf, u64 cval,
-                          size_t n, int L, const u64* qtab, const u64* delta, int N) {
-    const size_t total = n * 2 * L * N;
-    for (size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
-         idx += (size_t)gridDim.x * blockDim.x) {
-        const int k = (int)(idx % N);
-        const int i = (int)((idx / N) % L);
-        const int comp = (int)((idx / ((size_t)N * L)) & 1);
-        out[idx] = lin_word(cf.cc, cf.cx, cf.cy, cf.cz, cf.cp, cval, x, y, z, p, idx, comp, k, qtab[i], delta[i],
-                            delta[L + i]);
-    }
+template <int W>
+__global__ void __launch_bounds__(256) k_lincomb(u64* out, const u64* x, const u64* y, const u64* z, const u64* p, LinCoef cf,
+                                                 u64 cval, int L, const u64* qtab, const u64* delta, int logN) {
+    const Row<W> r(logN);
+    const uint32_t h = r.row / (uint32_t)L;
+    const int i = (int)(r.row - h * L);
+    store_words<W>(out + r.off, lin_words<W>(cf.cc, cf.cx, cf.cy, cf.cz, cf.cp, cval, x, y, z, p, r.off,
+                                             (h & 1) == 0 && r.k == 0, qtab[i], delta[i], delta[L + i]));
 }
 
 struct ScalarPairs {
     u64 w[BFHE_MAX_L], ws[BFHE_MAX_L];
 };
 
-__global__ void k_mul_scalar(const u64* a, u64* out, ScalarPairs sp, size_t n, int L, const u64* qtab, int N) {
-    const size_t total = n * 2 * L * N;
-    for (size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
-         idx += (size_t)gridDim.x * blockDim.x) {
-        const int i = (int)((idx / N) % L);
-        out[idx] = shoup(a[idx], sp.w[i], sp.ws[i], qtab[i]);
-    }
+template <int W>
+__global__ void __launch_bounds__(256) k_mul_scalar(const u64* a, u64* out, ScalarPairs sp, int L, const u64* qtab, int logN) {
+    const Row<W> r(logN);
+    const int i = (int)(r.row % (uint32_t)L);
+    const u64 q = qtab[i], w = sp.w[i], ws = sp.ws[i];
+    Words<W> t = load_words<W>(a + r.off);
+#pragma unroll
+    for (int j = 0; j < W; ++j) t.v[j] = shoup(t.v[j], w, ws, q);
+    store_words<W>(out + r.off, t);
 }
 
 // Listing 5: r = v[s-1]; r += r + v[i], i = s-2 .. 0
-__global__ void k_horner(const u64* bits, uint32_t s, u64* out, size_t n, int L, const u64* qtab, int N) {
-    const size_t words = n * 2 * L * N;
-    for (size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x; idx < words;
-         idx += (size_t)gridDim.x * blockDim.x) {
-        const u64 q = qtab[(idx / N) % L];
-        u64 r = bits[(size_t)(s - 1) * words + idx];
-        for (int i = (int)s - 2; i >= 0; --i) r = add_mod(r, add_mod(r, bits[(size_t)i * words + idx], q), q);
-        out[idx] = r;
+template <int W>
+__global__ void __launch_bounds__(256) k_horner(const u64* bits, uint32_t s, u64* out, size_t words, int L, const u64* qtab,
+                                                int logN) {
+    const Row<W> r(logN);
+    const u64 q = qtab[r.row % (uint32_t)L];
+    const u64* p = bits + (size_t)(s - 1) * words + r.off;
+    Words<W> acc = load_words<W>(p);
+#pragma unroll (W == 2 ? 8 : 4)
+    for (int i = (int)s - 2; i >= 0; --i) {
+        p -= words;
+        const Words<W> t = load_words<W>(p);
+#pragma unroll
+        for (int w = 0; w < W; ++w) acc.v[w] = add_mod(acc.v[w], add_mod(acc.v[w], t.v[w], q), q);
     }
+    store_words<W>(out + r.off, acc);
 }
 
-// gather gate operands: A[g] = wires[x], B[g] = wires[y] (MUX: wires[y] - wires[z])
-__global__ void k_gather_ops(u64* A, u64* B, const u64* wires, size_t ctw, const int32_t* table, int n_gates,
-                             int L, const u64* qtab, int N) {
-    const size_t total = (size_t)n_gates * ctw;
-    for (size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
-         idx += (size_t)gridDim.x * blockDim.x) {
-        const int g = (int)(idx / ctw);
-        const size_t o = idx % ctw;
-        const int32_t* e = table + 5 * g;
-        const u64 q = qtab[(o / N) % L];
-        A[idx] = wires[(size_t)e[1] * ctw + o];
-        const u64 yv = wires[(size_t)e[2] * ctw + o];
-        B[idx] = (e[0] & 0xff) == BFHE_MUX ? sub_mod(yv, wires[(size_t)e[3] * ctw + o], q) : yv;
+// gather gate operands: A[g] = wires[x], B[g] = wires[y] (MUX: wires[y] - wires[z]); rows: gate, then the wire's limbs
+template <int W>
+__global__ void __launch_bounds__(256) k_gather_ops(u64* A, u64* B, const u64* wires, uint32_t rows, const int32_t* table, int L,
+                                                    const u64* qtab, int logN) {
+    const Row<W> r(logN);
+    const uint32_t g = r.row / rows, lr = r.row - g * rows;
+    const size_t ctw = (size_t)rows << logN, o = ((size_t)lr << logN) + r.k;
+    const int32_t* e = table + 5 * g;
+    store_words<W>(A + r.off, load_words<W>(wires + (size_t)e[1] * ctw + o));
+    Words<W> y = load_words<W>(wires + (size_t)e[2] * ctw + o);
+    if ((e[0] & 0xff) == BFHE_MUX) {
+        const u64 q = qtab[lr % (uint32_t)L];
+        const Words<W> z = load_words<W>(wires + (size_t)e[3] * ctw + o);
+#pragma unroll
+        for (int w = 0; w < W; ++w) y.v[w] = sub_mod(y.v[w], z.v[w], q);
     }
+    store_words<W>(B + r.off, y);
 }
 
 // gate epilogue: wires[out] = lin(op)(x, y, z, prod[g]); entries g >= n_mul have no product
-__global__ void k_gate_epilogue(u64* wires, size_t ctw, const int32_t* table, int n_gates, int n_mul,
-                                const u64* prod, int L, const u64* qtab, const u64* delta, int N) {
-    const size_t total = (size_t)n_gates * ctw;
-    const size_t per_comp = (size_t)L * N;
-    for (size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
-         idx += (size_t)gridDim.x * blockDim.x) {
-        const int g = (int)(idx / ctw);
-        const size_t o = idx % ctw;
-        const int32_t* e = table + 5 * g;
-        const int op = e[0] & 0xff;
-        int cc, cx, cy, cz, cp;
-        if (op == BFHE_OP_MUL) {
-            cc = cx = cy = cz = 0;
-            cp = 1;
-        } else if (op == BFHE_OP_LIN) {
-            const int code = e[0] >> 8;
-            cc = code / 125 - 2;
-            cx = (code / 25) % 5 - 2;
-            cy = (code / 5) % 5 - 2;
-            cz = code % 5 - 2;
-            cp = 0;
-        } else {
-            const int* cf = c_gate_coef[op & 7];
-            cc = cf[0];
-            cx = cf[1];
-            cy = cf[2];
-            cz = cf[3];
-            cp = cf[4];
-        }
-        if (g >= n_mul) cp = 0;
-        const int i = (int)((o / N) % L);
-        const int k = (int)(o % N);
-        const int comp = (int)((o / per_comp) & 1);
-        const u64* x = wires + (size_t)e[1] * ctw;
-        const u64* y = wires + (size_t)e[2] * ctw;
-        const u64* z = wires + (size_t)e[3] * ctw;
-        const u64* p = g < n_mul ? prod + (size_t)g * ctw : nullptr;
-        wires[(size_t)e[4] * ctw + o] =
-            lin_word(cc, cx, cy, cz, cp, 1, x, y, z, p, o, comp, k, qtab[i], delta[i], delta[L + i]);
+template <int W>
+__global__ void __launch_bounds__(256) k_gate_epilogue(u64* wires, uint32_t rows, const int32_t* table, int n_mul, const u64* prod,
+                                                       int L, const u64* qtab, const u64* delta, int logN) {
+    const Row<W> r(logN);
+    const uint32_t g = r.row / rows, lr = r.row - g * rows;
+    const size_t ctw = (size_t)rows << logN, o = ((size_t)lr << logN) + r.k;
+    const int32_t* e = table + 5 * g;
+    const int op = e[0] & 0xff;
+    int cc, cx, cy, cz, cp;
+    if (op == BFHE_OP_MUL) {
+        cc = cx = cy = cz = 0;
+        cp = 1;
+    } else if (op == BFHE_OP_LIN) {
+        const int code = e[0] >> 8;
+        cc = code / 125 - 2;
+        cx = (code / 25) % 5 - 2;
+        cy = (code / 5) % 5 - 2;
+        cz = code % 5 - 2;
+        cp = 0;
+    } else {
+        const int* cf = c_gate_coef[op & 7];
+        cc = cf[0];
+        cx = cf[1];
+        cy = cf[2];
+        cz = cf[3];
+        cp = cf[4];
     }
+    if ((int)g >= n_mul) cp = 0;
+    const uint32_t h = lr / (uint32_t)L;
+    const int i = (int)(lr - h * L);
+    const u64* x = wires + (size_t)e[1] * ctw;
+    const u64* y = wires + (size_t)e[2] * ctw;
+    const u64* z = wires + (size_t)e[3] * ctw;
+    const u64* p = (int)g < n_mul ? prod + (size_t)g * ctw : nullptr;
+    store_words<W>(wires + (size_t)e[4] * ctw + o,
+                   lin_words<W>(cc, cx, cy, cz, cp, 1, x, y, z, p, o, (h & 1) == 0 && r.k == 0, qtab[i], delta[i], delta[L + i]));
+}
+
+// encrypt epilogue: ct[c][0] += Delta m + e1, ct[c][1] += e2; one block row per limb of c0, which does both components
+template <int W>
+__global__ void __launch_bounds__(256) k_enc_finish(u64* ct, const u64* M, const i64* e1, const i64* e2, int L, const u64* qtab,
+                                                    const u64* delta, int logN, u64 t, uint32_t* flags) {
+    const Row<W> r(logN);
+    const uint32_t c = r.row / (uint32_t)L, i = r.row - c * L;
+    const u64 q = qtab[i];
+    const size_t po = ((size_t)c << logN) + r.k;
+    const Words<W> m = load_words<W>(M + po);
+    const Words<W> a = load_words<W>(reinterpret_cast<const u64*>(e1) + po), b = load_words<W>(reinterpret_cast<const u64*>(e2) + po);
+    u64* p0 = ct + ((size_t)(2 * c * L + i) << logN) + r.k;
+    u64* p1 = p0 + ((size_t)L << logN);
+    Words<W> v0 = load_words<W>(p0), v1 = load_words<W>(p1);
+#pragma unroll
+    for (int w = 0; w < W; ++w) {
+        if (i == 0 && m.v[w] >= t) atomicOr(flags, BFHE_FLAG_PLAINTEXT);   // plaintext coefficients must be < t
+        const i64 x = (i64)a.v[w], y = (i64)b.v[w];
+        u64 v = add_mod(v0.v[w], shoup(m.v[w], delta[i], delta[L + i], q), q);
+        v0.v[w] = x >= 0 ? add_mod(v, (u64)x, q) : sub_mod(v, (u64)(-x), q);
+        v1.v[w] = y >= 0 ? add_mod(v1.v[w], (u64)y, q) : sub_mod(v1.v[w], (u64)(-y), q);
+    }
+    store_words<W>(p0, v0);
+    store_words<W>(p1, v1);
 }
 
 // integer-pipe probe: 8 independent lazy Shoup chains per thread
@@ -506,69 +560,53 @@ __global__ void k_probe_modmul(u64* out, uint32_t iters, u64 q, u64 w, u64 ws) {
 }
 
 // trivial ciphertexts (Delta bit_k(c_base + c), 0), layout [s][C][n][2][L][N]
-__global__ void k_trivial_bits(u64* out, uint32_t s, u64 c_base, const u64* cbp, int C, size_t n, int L,
-                               const u64* delta, int N) {
+template <int W>
+__global__ void __launch_bounds__(256) k_trivial_bits(u64* out, u64 c_base, const u64* cbp, uint32_t C, uint32_t n, int L,
+                                                      const u64* delta, int logN) {
+    const Row<W> r(logN);
     if (cbp) c_base = *cbp;
-    const size_t ctw = (size_t)2 * L * N;
-    const size_t total = (size_t)s * C * n * ctw;
-    for (size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
-         idx += (size_t)gridDim.x * blockDim.x) {
-        const size_t o = idx % ctw;
-        const size_t rest = idx / ctw;
-        const int c = (int)((rest / n) % C);
-        const int kbit = (int)(rest / (n * C));
-        const int i = (int)(o / N);   // < L only for c0
-        u64 v = 0;
-        if (o < (size_t)L * N && (o % N) == 0 && (((c_base + c) >> kbit) & 1)) v = delta[i];
-        out[idx] = v;
-    }
+    const uint32_t h = r.row / (uint32_t)L, i = r.row - h * L;   // h: (bit, c, n, component)
+    const uint32_t cn = (h >> 1) / n, kbit = cn / C, c = cn - kbit * C;
+    Words<W> t{};
+    if ((h & 1) == 0 && r.k == 0 && (((c_base + c) >> kbit) & 1)) t.v[0] = delta[i];
+    store_words<W>(out + r.off, t);
 }
 
 // bits[k][i] += sum over c of src (PAPER: src [s][C][n]; SELECT: src [C][n], only if bit k of c)
-__global__ void k_accumulate(u64* bits, const u64* src, uint32_t s, u64 c_base, const u64* cbp, int C, size_t n,
-                             int select, int L, const u64* qtab, int N) {
+template <int W>
+__global__ void __launch_bounds__(256) k_accumulate(u64* bits, const u64* src, uint32_t rows, u64 c_base, const u64* cbp, int C,
+                                                    int select, int L, const u64* qtab, int logN) {
+    const Row<W> r(logN);
     if (cbp) c_base = *cbp;
-    const size_t ctw = (size_t)2 * L * N;
-    const size_t words = n * ctw;
-    const size_t total = (size_t)s * words;
-    for (size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
-         idx += (size_t)gridDim.x * blockDim.x) {
-        const int kbit = (int)(idx / words);
-        const size_t w = idx % words;
-        const u64 q = qtab[(w / N) % L];
-        u64 acc = bits[idx];
-        for (int c = 0; c < C; ++c) {
-            if (select) {
-                if (((c_base + c) >> kbit) & 1) acc = add_mod(acc, src[(size_t)c * words + w], q);
-            } else {
-                acc = add_mod(acc, src[((size_t)kbit * C + c) * words + w], q);
-            }
-        }
-        bits[idx] = acc;
+    const uint32_t kbit = r.row / rows, lr = r.row - kbit * rows;
+    const size_t words = (size_t)rows << logN, w0 = ((size_t)lr << logN) + r.k;
+    const u64 q = qtab[lr % (uint32_t)L];
+    Words<W> acc = load_words<W>(bits + r.off);
+    const u64* p = src + w0 + (select ? 0 : (size_t)kbit * C * words);
+#pragma unroll 4
+    for (int c = 0; c < C; ++c, p += words) {
+        if (select && !(((c_base + c) >> kbit) & 1)) continue;
+        const Words<W> t = load_words<W>(p);
+#pragma unroll
+        for (int w = 0; w < W; ++w) acc.v[w] = add_mod(acc.v[w], t.v[w], q);
     }
+    store_words<W>(bits + r.off, acc);
 }
 
 // out[c][i] = x[i] - (c_base + c)   (layout [C][n])
-__global__ void k_sub_const_chains(const u64* x, u64* out, u64 c_base, const u64* cbp, int C, size_t n, int L,
-                                   const u64* qtab, const u64* delta, u64 t, int N) {
+template <int W>
+__global__ void __launch_bounds__(256) k_sub_const_chains(const u64* x, u64* out, uint32_t rows, u64 c_base, const u64* cbp, int L,
+                                                          const u64* qtab, const u64* delta, u64 t, int logN) {
+    const Row<W> r(logN);
     if (cbp) c_base = *cbp;
-    const size_t ctw = (size_t)2 * L * N;
-    const size_t words = n * ctw;
-    const size_t total = (size_t)C * words;
-    for (size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
-         idx += (size_t)gridDim.x * blockDim.x) {
-        const int c = (int)(idx / words);
-        const size_t w = idx % words;
-        const size_t o = w % ctw;
-        u64 v = x[w];
-        if (o < (size_t)L * N && (o % N) == 0) {
-            const int i = (int)(o / N);
-            const u64 q = qtab[i];
-            const u64 cv = (c_base + c) % t;
-            v = sub_mod(v, shoup(cv, delta[i], delta[L + i], q), q);
-        }
-        out[idx] = v;
+    const uint32_t c = r.row / rows, lr = r.row - c * rows;
+    const uint32_t h = lr / (uint32_t)L, i = lr - h * L;
+    Words<W> v = load_words<W>(x + ((size_t)lr << logN) + r.k);
+    if ((h & 1) == 0 && r.k == 0) {
+        const u64 q = qtab[i];
+        v.v[0] = sub_mod(v.v[0], shoup((c_base + c) % t, delta[i], delta[L + i], q), q);
     }
+    store_words<W>(out + r.off, v);
 }
 
 // one device word (the candidate base read by a replayed mod_to_bits tile)
@@ -671,10 +709,19 @@ int launch_permute(const bfhe_ctx* ctx, const u64* in, u64* out, int n, int scat
     return BFHE_OK;
 }
 
+// one block per 256 W words of each row; two words per thread when every buffer is 16-byte aligned
+#define LAUNCH_ROWS(kern, wide, rows, ...)                                                                     \
+    do {                                                                                                       \
+        const size_t _rows = (rows);                                                                           \
+        if (wide) kern<2><<<(unsigned)(_rows << (ctx->logN - 9)), TPB, 0, st>>>(__VA_ARGS__);                  \
+        else kern<1><<<(unsigned)(_rows << (ctx->logN - 8)), TPB, 0, st>>>(__VA_ARGS__);                       \
+        BFHE_LAUNCH_CHECK(#kern);                                                                              \
+    } while (0)
+
 int launch_enc_finish(const bfhe_ctx* ctx, u64* ct, const u64* M, const i64* e1, const i64* e2, int n,
                       cudaStream_t st) {
-    LAUNCH(k_enc_finish, (size_t)n * ctx->L * ctx->N, ct, M, e1, e2, n, (int)ctx->L, ctx->tab.q, ctx->d_delta_q,
-           (int)ctx->N, ctx->t, ctx->d_flags);
+    LAUNCH_ROWS(k_enc_finish, aligned16(ct) && aligned16(M) && aligned16(e1) && aligned16(e2), (size_t)n * ctx->L, ct, M, e1,
+                e2, (int)ctx->L, ctx->tab.q, ctx->d_delta_q, (int)ctx->logN, ctx->t, ctx->d_flags);
     return BFHE_OK;
 }
 
@@ -687,8 +734,10 @@ int launch_neg_add_small(const bfhe_ctx* ctx, const u64* as, const i64* e, u64* 
 
 int launch_lincomb(const bfhe_ctx* ctx, u64* out, const u64* x, const u64* y, const u64* z, const u64* p,
                    LinCoef cf, u64 cval, size_t n, cudaStream_t st) {
-    LAUNCH(k_lincomb, n * ctx->ct_words(), out, x, y, z, p, cf, cval, n, (int)ctx->L, ctx->tab.q, ctx->d_delta_q,
-           (int)ctx->N);
+    const bool wide = aligned16(out) && (!cf.cx || aligned16(x)) && (!cf.cy || aligned16(y)) && (!cf.cz || aligned16(z)) &&
+                      (!cf.cp || aligned16(p));
+    LAUNCH_ROWS(k_lincomb, wide, n * 2 * ctx->L, out, x, y, z, p, cf, cval, (int)ctx->L, ctx->tab.q, ctx->d_delta_q,
+                (int)ctx->logN);
     return BFHE_OK;
 }
 
@@ -700,54 +749,52 @@ int launch_mul_scalar(const bfhe_ctx* ctx, const u64* a, u64 c, u64* out, size_t
         sp.w[i] = w;
         sp.ws[i] = (u64)(((u128)w << 64) / q);
     }
-    LAUNCH(k_mul_scalar, n * ctx->ct_words(), a, out, sp, n, (int)ctx->L, ctx->tab.q, (int)ctx->N);
+    LAUNCH_ROWS(k_mul_scalar, aligned16(a) && aligned16(out), n * 2 * ctx->L, a, out, sp, (int)ctx->L, ctx->tab.q,
+                (int)ctx->logN);
     return BFHE_OK;
 }
 
 int launch_horner(const bfhe_ctx* ctx, const u64* bits, uint32_t s, u64* out, size_t n, cudaStream_t st) {
-    LAUNCH(k_horner, n * ctx->ct_words(), bits, s, out, n, (int)ctx->L, ctx->tab.q, (int)ctx->N);
+    LAUNCH_ROWS(k_horner, aligned16(bits) && aligned16(out), n * 2 * ctx->L, bits, s, out, n * ctx->ct_words(), (int)ctx->L,
+                ctx->tab.q, (int)ctx->logN);
     return BFHE_OK;
 }
 
 int launch_gather(const bfhe_ctx* ctx, u64* dst, const u64* wires, size_t n, const int32_t* table, int n_gates,
-                  int field, int sub_field, cudaStream_t st) {
-    // field/sub_field are unused by this layout: dst holds A then B ([2][n_gates][n] ciphertexts)
-    (void)field;
-    (void)sub_field;
+                  cudaStream_t st) {
+    // dst holds A then B ([2][n_gates][n] ciphertexts)
     const size_t ctw = n * ctx->ct_words();
-    u64* A = dst;
-    u64* B = dst + (size_t)n_gates * ctw;
-    LAUNCH(k_gather_ops, (size_t)n_gates * ctw, A, B, wires, ctw, table, n_gates, (int)ctx->L, ctx->tab.q,
-           (int)ctx->N);
+    LAUNCH_ROWS(k_gather_ops, aligned16(dst) && aligned16(wires), (size_t)n_gates * n * 2 * ctx->L, dst,
+                dst + (size_t)n_gates * ctw, wires, (uint32_t)(n * 2 * ctx->L), table, (int)ctx->L, ctx->tab.q,
+                (int)ctx->logN);
     return BFHE_OK;
 }
 
 int launch_gate_epilogue(const bfhe_ctx* ctx, u64* wires, size_t n, const int32_t* table, int n_gates,
                          const u64* prod, int n_mul, cudaStream_t st) {
-    const size_t ctw = n * ctx->ct_words();
-    LAUNCH(k_gate_epilogue, (size_t)n_gates * ctw, wires, ctw, table, n_gates, n_mul, prod, (int)ctx->L, ctx->tab.q,
-           ctx->d_delta_q, (int)ctx->N);
+    LAUNCH_ROWS(k_gate_epilogue, aligned16(wires) && aligned16(prod), (size_t)n_gates * n * 2 * ctx->L, wires,
+                (uint32_t)(n * 2 * ctx->L), table, n_mul, prod, (int)ctx->L, ctx->tab.q, ctx->d_delta_q, (int)ctx->logN);
     return BFHE_OK;
 }
 
 int launch_trivial_bits(const bfhe_ctx* ctx, u64* out, uint32_t s, u64 c_base, const u64* cbp, int C, size_t n,
                         cudaStream_t st) {
-    LAUNCH(k_trivial_bits, (size_t)s * C * n * ctx->ct_words(), out, s, c_base, cbp, C, n, (int)ctx->L, ctx->d_delta_q,
-           (int)ctx->N);
+    LAUNCH_ROWS(k_trivial_bits, aligned16(out), (size_t)s * C * n * 2 * ctx->L, out, c_base, cbp, (uint32_t)C, (uint32_t)n,
+                (int)ctx->L, ctx->d_delta_q, (int)ctx->logN);
     return BFHE_OK;
 }
 
 int launch_accumulate(const bfhe_ctx* ctx, u64* bits, const u64* src, uint32_t s, u64 c_base, const u64* cbp, int C,
                       size_t n, int select, cudaStream_t st) {
-    LAUNCH(k_accumulate, (size_t)s * n * ctx->ct_words(), bits, src, s, c_base, cbp, C, n, select, (int)ctx->L, ctx->tab.q,
-           (int)ctx->N);
+    LAUNCH_ROWS(k_accumulate, aligned16(bits) && aligned16(src), (size_t)s * n * 2 * ctx->L, bits, src,
+                (uint32_t)(n * 2 * ctx->L), c_base, cbp, C, select, (int)ctx->L, ctx->tab.q, (int)ctx->logN);
     return BFHE_OK;
 }
 
 int launch_sub_const_chains(const bfhe_ctx* ctx, const u64* x, u64* out, u64 c_base, const u64* cbp, int C, size_t n,
                             cudaStream_t st) {
-    LAUNCH(k_sub_const_chains, (size_t)C * n * ctx->ct_words(), x, out, c_base, cbp, C, n, (int)ctx->L, ctx->tab.q,
-           ctx->d_delta_q, ctx->t, (int)ctx->N);
+    LAUNCH_ROWS(k_sub_const_chains, aligned16(x) && aligned16(out), (size_t)C * n * 2 * ctx->L, x, out,
+                (uint32_t)(n * 2 * ctx->L), c_base, cbp, (int)ctx->L, ctx->tab.q, ctx->d_delta_q, ctx->t, (int)ctx->logN);
     return BFHE_OK;
 }
 

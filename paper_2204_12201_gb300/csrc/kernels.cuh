@@ -51,7 +51,7 @@ int launch_mul_scalar(const bfhe_ctx* ctx, const u64* a, u64 c, u64* out, size_t
 int launch_horner(const bfhe_ctx* ctx, const u64* bits, uint32_t s, u64* out, size_t n, cudaStream_t st);
 // gate table helpers
 int launch_gather(const bfhe_ctx* ctx, u64* dst, const u64* wires, size_t n, const int32_t* table, int n_gates,
-                  int field, int sub_field, cudaStream_t st);
+                  cudaStream_t st);
 int launch_gate_epilogue(const bfhe_ctx* ctx, u64* wires, size_t n, const int32_t* table, int n_gates,
                          const u64* prod, int n_mul, cudaStream_t st);
 // mod_to_bits helpers; the candidate base is c_base, or the device word *cbp when cbp is not null
