@@ -18,7 +18,7 @@ OBJDIR = os.path.join(ROOT, "_build")
 # (object, source, defines): the kernels of ntt.cu and ext_pm.cu compile as several objects in parallel
 UNITS = [("host", "host.cu", []), ("kernels", "kernels.cu", []), ("ext", "ext.cu", []), ("api", "api.cu", [])]
 UNITS += [("ext_pm%d" % p, "ext_pm.cu", ["-DBFHE_EXT_PM_PART=%d" % p]) for p in range(5)]
-UNITS += [("ntt%d" % p, "ntt.cu", ["-DBFHE_NTT_PART=%d" % p]) for p in range(4)]
+UNITS += [("ntt%d" % p, "ntt.cu", ["-DBFHE_NTT_PART=%d" % p]) for p in range(5)]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC", "-Xcompiler", "-O2"]
 

@@ -315,6 +315,14 @@ extern "C" int bfhe_export_keys(bfhe_ctx* c, int64_t* sk, uint64_t* pk, uint64_t
 
 namespace {
 
+// one polynomial of small (signed) words in, all its limbs out
+NttIO ntt_small(const void* in, u64* out, size_t L, size_t N) {
+    NttIO io = ntt_io((const u64*)in, out, L, N);
+    io.in_os = N;
+    io.in_ls = 0;
+    return io;
+}
+
 // (Delta M + pk0 u + e1, pk1 u + e2) for plaintext polynomials M [n][N] (coefficients < t);
 // scratch: u/e1/e2 [3][n][N], U [n][L][N]
 int encrypt_core(bfhe_ctx* c, const u64* M, size_t n, uint64_t seed, u64* ct_out, u64* scratch, cudaStream_t st) {
@@ -326,11 +334,24 @@ int encrypt_core(bfhe_ctx* c, const u64* M, size_t n, uint64_t seed, u64* ct_out
     RC(launch_sample_small(c, u, (int)n, seed, P_ENC_U, 0, 0, st));
     RC(launch_sample_small(c, e1, (int)n, seed, P_ENC_E1, 0, 1, st));
     RC(launch_sample_small(c, e2, (int)n, seed, P_ENC_E2, 0, 1, st));
-    RC(launch_spread(c, u, U, (int)n, (int)L, c->mapQ(), st));
-    RC(launch_ntt_fwd(c, ntt_io(U, U, L, N), (int)n, (int)L, c->mapQ(), st));
-    PwStrides s{L * N, 0, 0, L * N, 2 * L * N, L * N};
-    RC(launch_pointwise(c, U, c->d_pk_ntt, ct_out, (int)n, 2, (int)L, c->mapQ(), s, st));
-    RC(launch_ntt_inv(c, ntt_io(ct_out, ct_out, L, N), (int)(2 * n), (int)L, c->mapQ(), 1, st));
+    if (c->pm) {
+        // the transform takes the signed ternary words as they are, the inverse multiplies by the key as it loads
+        RC(launch_ntt_fwd(c, ntt_small(u, U, L, N), (int)n, (int)L, c->mapQ(), st, 1));
+        NttIO io = ntt_io(U, ct_out, L, N);
+        io.n_inner = 2;
+        io.in_is = 0;
+        io.out_os = 2 * L * N;
+        io.out_is = L * N;
+        io.mul = c->d_pk_ntt;
+        io.mul_is = L * N;
+        RC(launch_ntt_inv(c, io, (int)(2 * n), (int)L, c->mapQ(), 0, st));
+    } else {
+        RC(launch_spread(c, u, U, (int)n, (int)L, c->mapQ(), st));
+        RC(launch_ntt_fwd(c, ntt_io(U, U, L, N), (int)n, (int)L, c->mapQ(), st));
+        PwStrides s{L * N, 0, 0, L * N, 2 * L * N, L * N};
+        RC(launch_pointwise(c, U, c->d_pk_ntt, ct_out, (int)n, 2, (int)L, c->mapQ(), s, st));
+        RC(launch_ntt_inv(c, ntt_io(ct_out, ct_out, L, N), (int)(2 * n), (int)L, c->mapQ(), 1, st));
+    }
     RC(launch_enc_finish(c, ct_out, M, e1, e2, (int)n, st));
     return BFHE_OK;
 }
@@ -348,10 +369,17 @@ int decrypt_core(bfhe_ctx* c, const u64* ct, size_t n, u64* M, u64* V, cudaStrea
     io.out_os = L * N;
     io.out_is = 0;
     io.out_ls = N;
-    RC(launch_ntt_fwd(c, io, (int)n, (int)L, c->mapQ(), st));
-    PwStrides s{L * N, 0, 0, 0, L * N, 0};
-    RC(launch_pointwise(c, V, c->d_sk_ntt, V, (int)n, 1, (int)L, c->mapQ(), s, st));
-    RC(launch_ntt_inv(c, ntt_io(V, V, L, N), (int)n, (int)L, c->mapQ(), 1, st));
+    if (c->pm) {
+        RC(launch_ntt_fwd(c, io, (int)n, (int)L, c->mapQ(), st, 1));
+        NttIO iv = ntt_io(V, V, L, N);
+        iv.mul = c->d_sk_ntt;
+        RC(launch_ntt_inv(c, iv, (int)n, (int)L, c->mapQ(), 0, st));
+    } else {
+        RC(launch_ntt_fwd(c, io, (int)n, (int)L, c->mapQ(), st));
+        PwStrides s{L * N, 0, 0, 0, L * N, 0};
+        RC(launch_pointwise(c, V, c->d_sk_ntt, V, (int)n, 1, (int)L, c->mapQ(), s, st));
+        RC(launch_ntt_inv(c, ntt_io(V, V, L, N), (int)n, (int)L, c->mapQ(), 1, st));
+    }
     RC(launch_dec_finish(c, V, ct, M, (int)n, st));
     return BFHE_OK;
 }
@@ -480,12 +508,24 @@ extern "C" int bfhe_mul_plain(bfhe_ctx* c, const uint64_t* a, const uint64_t* pl
     u64* CT = PT + n * L * N;
     RC(launch_permute(c, plain, M, (int)n, 1, st));
     RC(launch_ntt_inv(c, ntt_io(M, M, 1, N), (int)n, 1, c->mapT(), 0, st));
-    RC(launch_spread(c, (const i64*)M, PT, (int)n, (int)L, c->mapQ(), st));
-    RC(launch_ntt_fwd(c, ntt_io(PT, PT, L, N), (int)n, (int)L, c->mapQ(), st));
-    RC(launch_ntt_fwd(c, ntt_io(a, CT, L, N), (int)(2 * n), (int)L, c->mapQ(), st));
-    PwStrides s{2 * L * N, L * N, L * N, 0, 2 * L * N, L * N};
-    RC(launch_pointwise(c, CT, PT, out, (int)n, 2, (int)L, c->mapQ(), s, st));
-    RC(launch_ntt_inv(c, ntt_io(out, out, L, N), (int)(2 * n), (int)L, c->mapQ(), 1, st));
+    if (c->pm) {
+        RC(launch_ntt_fwd(c, ntt_small(M, PT, L, N), (int)n, (int)L, c->mapQ(), st, 1));
+        RC(launch_ntt_fwd(c, ntt_io(a, CT, L, N), (int)(2 * n), (int)L, c->mapQ(), st, 1));
+        NttIO io = ntt_io(CT, out, L, N);
+        io.n_inner = 2;
+        io.in_os = io.out_os = 2 * L * N;
+        io.in_is = io.out_is = L * N;
+        io.mul = PT;
+        io.mul_os = L * N;
+        RC(launch_ntt_inv(c, io, (int)(2 * n), (int)L, c->mapQ(), 0, st));
+    } else {
+        RC(launch_spread(c, (const i64*)M, PT, (int)n, (int)L, c->mapQ(), st));
+        RC(launch_ntt_fwd(c, ntt_io(PT, PT, L, N), (int)n, (int)L, c->mapQ(), st));
+        RC(launch_ntt_fwd(c, ntt_io(a, CT, L, N), (int)(2 * n), (int)L, c->mapQ(), st));
+        PwStrides s{2 * L * N, L * N, L * N, 0, 2 * L * N, L * N};
+        RC(launch_pointwise(c, CT, PT, out, (int)n, 2, (int)L, c->mapQ(), s, st));
+        RC(launch_ntt_inv(c, ntt_io(out, out, L, N), (int)(2 * n), (int)L, c->mapQ(), 1, st));
+    }
     c->counts[3] += n;
     return BFHE_OK;
 }

@@ -163,6 +163,24 @@ __device__ __forceinline__ u64 pm_canon(u64 x, u64 q, int b, uint32_t d) {
     const u64 y = pm_lazy(x, q, b, d);
     return y >= q ? y - q : y;
 }
+// a b mod q, canonical, for two run-time factors below 2^(bits+1): the 128-bit product folded three times (eight wide
+// multiplies against Montgomery's ten and their carries)
+__device__ __forceinline__ u64 pm_mul_var(u64 a, u64 b, u64 q, int bits, uint32_t d) {
+    const uint32_t a0 = (uint32_t)a, a1 = (uint32_t)(a >> 32), b0 = (uint32_t)b, b1 = (uint32_t)(b >> 32);
+    const u64 lo = (u64)a0 * b0;
+    u64 m = mad_wide_u(a1, b0, lo >> 32);      // below 2^57 + 2^32
+    m = mad_wide_u(a0, b1, m);
+    const u64 top = mad_wide_u(a1, b1, m >> 32);
+    const int s = bits - 32;
+    // product = H 2^bits + (m mod 2^s) 2^32 + lo: H = h1 2^32 + h0
+    const uint32_t h0 = __funnelshift_r((uint32_t)m, (uint32_t)top, s), h1 = (uint32_t)(top >> s);
+    const u64 g = (u64)h1 * d;                 // weight 2^32: g = (g >> s) 2^s + f, 2^(s + 32) = 2^bits
+    u64 r = ((u64)(((uint32_t)m & ((1u << s) - 1u))) << 32) | (uint32_t)lo;
+    r += (u64)((uint32_t)g & ((1u << s) - 1u)) << 32;
+    r = mad_wide_u(h0, d, r);
+    r = mad_wide_u((uint32_t)(g >> s), d, r);  // below 2^60
+    return pm_canon(r, q, bits, d);
+}
 // host: the table entry of w, cut at bit k (b - 30 for pm_mul)
 inline void pm_entry(u64 w, u64 q, int k, u64* x, u64* y) {
     const u64 m = ((u64)1 << k) - 1, v = (u64)(((u128)w << 32) % q);
@@ -218,6 +236,14 @@ struct PmSum {
     u64 guard = 0;                    // bound of 2^b |sum y_i / s_i - sum y_i / 2^b|
 };
 
+// Host constants of decryption's last step in the same arithmetic, for t below 2^26: t (Q/q_i)^-1 mod q_i as (l, h) of it
+// and of 2^32 times it, 1/q_i and 2^hs/q_i mod t
+struct PmDec {
+    std::vector<uint32_t> w, d, c, c2;   // [n][4], [n], [n], [n]
+    std::vector<u64> q;
+    u64 guard = 0;
+};
+
 // Device-side prime tables of a context, by prime index
 // (0..L-1 data, L..L+alpha-1 special, L+alpha..L+alpha+K-1 auxiliary, last: t).  The pairs of tw, twl, itw and
 // twist are pm_mul's entries for the moduli of a context with pm set, (w, Shoup(w)) otherwise and always for t.
@@ -256,6 +282,7 @@ struct bfhe_ctx {
     // pm contexts of at most 16 data primes: the input extension, scale-and-round's two sums and its twist table
     // [L + K][N] (data: t R N^-1 psi^-k (Q/q_i)^-1; auxiliary: t R N^-1 psi^-k Q^-1 (B/b_j)^-1; words cut at b - 28)
     PmSum pm_up, pm_toB, pm_toQ;
+    PmDec pm_dec;
     const ulonglong2* d_xtw = nullptr;
     // Shoup pair tables: p[i] = w_i, p[n + i] = ws_i
     const u64* d_tmod = nullptr;    // [nP] [t]_{prime}
@@ -372,6 +399,10 @@ struct NttIO {
     // [outer][2][src_limbs][N] of which inner & 1 selects the polynomial (the multiply's inputs, which need no copy)
     const u64* src[2] = {nullptr, nullptr};
     int src_limbs = 0;
+    // inverse only, pm contexts, canonical outputs: every input word is first multiplied by the word of the same limb
+    // and index of mul (poly (outer, inner) at outer mul_os + inner mul_is, limbs N words apart); factors below 2q
+    const u64* mul = nullptr;
+    size_t mul_os = 0, mul_is = 0;
 };
 // contiguous [n_polys][n_limbs][N] in and out
 inline NttIO ntt_io(const u64* in, u64* out, size_t n_limbs, size_t N) {

@@ -553,6 +553,8 @@ int launch_moddown(const bfhe_ctx* ctx, const u64* W, const u64* C3, u64* out, i
 }
 
 int launch_dec_finish(const bfhe_ctx* ctx, const u64* V, const u64* ct, u64* M, int n, cudaStream_t st) {
+    // (64-bit sums of 26-bit words mod t)
+    if (ctx->use_pm_ext() && ctx->t < ((u64)1 << 26)) return launch_dec_pm(ctx, V, ct, M, n, st);
     SWITCH_L(ctx->L, run_dec_finish, ctx, V, ct, M, n, st)
     if (ctx->L > BFHE_MAX_L) return set_error(BFHE_EINVAL, "unsupported number of data primes");
     LAUNCH(k_dec_finish_n, (size_t)n * ctx->N, V, ct, M, n, ctx->ext_Qt, ctx->d_tmod, (int)ctx->nP, ctx->Qinv_t,

@@ -352,6 +352,93 @@ __global__ void __launch_bounds__(256, 2)
     }
 }
 
+// decryption's last step for t < 2^26: with y_i = [t (c0 + c1 s) (Q/q_i)^-1]_{q_i} and v nearest to sum y_i / q_i, the
+// centred [t x]_Q is sum y_i (Q/q_i) - v Q and the plaintext -[t x]_Q / Q = v - sum y_i / q_i mod t.
+template <int NS>
+struct DecTab {
+    uint4 w[NS];
+    u64 q[NS];
+    uint32_t d[NS], c[NS], c2[NS];
+    u64 guard, t, mu, Qinv_t;
+};
+
+__device__ __noinline__ u64 dec_exact(const u64* V, const u64* c0, int N, ExtDesc e, const u64* tmod, int nP, u64 Qinv_t) {
+    const int ns = e.n_src;
+    u64 r[NMAX], v[NMAX];
+    for (int i = 0; i < ns; ++i)
+        r[i] = shoup(add_mod(V[(size_t)i * N], c0[(size_t)i * N], e.src_q[i]), tmod[i], tmod[nP + i], e.src_q[i]);
+    const bool neg = garner_n(r, e, v, ns);
+    const u64 t = e.dst_q[0], rho = ext_eval_n(v, neg, e, 0, ns, true);
+    return ((rho == 0 ? 0 : t - rho) * Qinv_t) % t;
+}
+
+template <int NS>
+__global__ void __launch_bounds__(256, 4)
+    k_dec_pm(const u64* __restrict__ V, const u64* __restrict__ ct, u64* __restrict__ M, int n, int logN, int b, ExtDesc ext,
+             const u64* tmod, int nP, uint32_t* flags, const __grid_constant__ DecTab<NS> p) {
+    const int k = b - 28, hs = (b + 2) >> 1;
+    const size_t total = (size_t)n << logN;
+    for (size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
+         idx += (size_t)gridDim.x * blockDim.x) {
+        const int kk = (int)(idx & ((1u << logN) - 1u));
+        const size_t c = idx >> logN;
+        const u64* vp = V + (c * NS << logN) + kk;
+        const u64* cp = ct + (c * 2 * NS << logN) + kk;
+        u64 x[NS];
+        bool bad = false;
+#pragma unroll
+        for (int i = 0; i < NS; ++i) {
+            const u64 c0 = cp[(size_t)i << logN];
+            bad |= c0 >= p.q[i];
+            x[i] = vp[(size_t)i << logN] + c0;
+        }
+        if (bad) atomicOr(flags, BFHE_FLAG_RESIDUE);
+        i64 sum = 0;
+        u64 z = p.t << 26;   // the digits may be slightly negative
+#pragma unroll
+        for (int i = 0; i < NS; ++i) {
+            const uint32_t a0 = (uint32_t)x[i];
+            const int a1 = (int)(x[i] >> 32);
+            u64 Q = (u64)a0 * p.w[i].y;
+            Q = mad_wide_s(a1, (int)p.w[i].w, Q);
+            u64 P = shl_word((uint32_t)Q, k);
+            P = mad_wide_u(a0, p.w[i].x, P);
+            P = mad_wide_s(a1, (int)p.w[i].z, P);
+            P = mad_wide_s((int)(Q >> 32), (int)(p.d[i] << 4), P);
+            const u64 y = pm_fold(P, b, p.d[i]);
+            sum = (i64)add64((u64)sum, y);
+            z = mad_wide_u((uint32_t)y & ((1u << hs) - 1u), p.c[i], z);
+            z = mad_wide_s((int)__funnelshift_r((uint32_t)y, (uint32_t)(y >> 32), hs), (int)p.c2[i], z);
+        }
+        int v;
+        if (!round_sum(sum, b, p.guard, v)) {
+            M[idx] = dec_exact(vp, cp, 1 << logN, ext, tmod, nP, p.Qinv_t);
+            continue;
+        }
+        M[idx] = reduce64((u64)((i64)v + (i64)(64 * p.t) - (i64)reduce64(z, p.t, p.mu)), p.t, p.mu);
+    }
+}
+
+template <int NS>
+int run_dec_pm(const bfhe_ctx* ctx, const u64* V, const u64* ct, u64* M, int n, cudaStream_t st) {
+    const PmDec& h = ctx->pm_dec;
+    DecTab<NS> t{};
+    for (int i = 0; i < NS; ++i) {
+        t.w[i] = make_uint4(h.w[4 * i], h.w[4 * i + 1], h.w[4 * i + 2], h.w[4 * i + 3]);
+        t.q[i] = h.q[i];
+        t.d[i] = h.d[i];
+        t.c[i] = h.c[i];
+        t.c2[i] = h.c2[i];
+    }
+    t.guard = h.guard;
+    t.t = ctx->t;
+    t.mu = (u64)(((u128)1 << 64) / ctx->t);
+    t.Qinv_t = ctx->Qinv_t;
+    LAUNCH(k_dec_pm<NS>, (size_t)n * ctx->N, V, ct, M, n, (int)ctx->logN, (int)ctx->prime_bits, ctx->ext_Qt, ctx->d_tmod,
+           (int)ctx->nP, ctx->d_flags, t);
+    return BFHE_OK;
+}
+
 template <int NS>
 int run_modup_pm(const bfhe_ctx* ctx, const u64* A, const u64* B, u64* X, int n, int slots, cudaStream_t st) {
     LAUNCH(k_modup_pm<NS>, (size_t)n * slots * ctx->N, A, B, X, n, slots, (int)ctx->logN, (int)ctx->prime_bits,
@@ -427,10 +514,18 @@ int PM_NAME(scale_pm)(const bfhe_ctx* ctx, const u64* X, u64* C3, int n, cudaStr
     }
 }
 
+int PM_NAME(dec_pm)(const bfhe_ctx* ctx, const u64* V, const u64* ct, u64* M, int n, cudaStream_t st) {
+    switch (ctx->L) {
+        PM_CASES(run_dec_pm, ctx, V, ct, M, n, st)
+        default: return set_error(BFHE_EINVAL, "unsupported number of data primes");
+    }
+}
+
 #if BFHE_EXT_PM_PART == 0
 #define PM_DECLARE(p)                                                                                               \
     int modup_pm_##p(const bfhe_ctx* ctx, const u64* A, const u64* B, u64* X, int n, int slots, cudaStream_t st);  \
-    int scale_pm_##p(const bfhe_ctx* ctx, const u64* X, u64* C3, int n, cudaStream_t st, u64* tmp);
+    int scale_pm_##p(const bfhe_ctx* ctx, const u64* X, u64* C3, int n, cudaStream_t st, u64* tmp);                 \
+    int dec_pm_##p(const bfhe_ctx* ctx, const u64* V, const u64* ct, u64* M, int n, cudaStream_t st);
 PM_DECLARE(1) PM_DECLARE(2) PM_DECLARE(3) PM_DECLARE(4)
 
 static int pm_part(uint32_t L) { return L <= 8 ? 0 : L <= 12 ? 1 : L <= 14 ? 2 : L == 15 ? 3 : 4; }
@@ -452,6 +547,16 @@ int launch_scale_pm(const bfhe_ctx* ctx, const u64* X, u64* C3, int n, cudaStrea
         case 2: return scale_pm_2(ctx, X, C3, n, st, tmp);
         case 3: return scale_pm_3(ctx, X, C3, n, st, tmp);
         default: return scale_pm_4(ctx, X, C3, n, st, tmp);
+    }
+}
+
+int launch_dec_pm(const bfhe_ctx* ctx, const u64* V, const u64* ct, u64* M, int n, cudaStream_t st) {
+    switch (pm_part(ctx->L)) {
+        case 0: return dec_pm_0(ctx, V, ct, M, n, st);
+        case 1: return dec_pm_1(ctx, V, ct, M, n, st);
+        case 2: return dec_pm_2(ctx, V, ct, M, n, st);
+        case 3: return dec_pm_3(ctx, V, ct, M, n, st);
+        default: return dec_pm_4(ctx, V, ct, M, n, st);
     }
 }
 #endif

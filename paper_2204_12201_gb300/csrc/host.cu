@@ -686,6 +686,20 @@ extern "C" int bfhe_ctx_create(const bfhe_params* prm, int device, bfhe_ctx** ou
         c->pm_up = pm_sum(Qp, Bp, b, y_up, up, v_up);
         c->pm_toB = pm_sum(Qp, Bp, b, y_sc, toB, v_toB);
         c->pm_toQ = pm_sum(Bp, Qp, b, y_sc, toQ, v_toQ);
+        c->pm_dec.guard = c->pm_toB.guard;   // the same sources and digits
+        for (uint32_t i = 0; i < L; ++i) {
+            const u64 m = Qp[i], ci = invmod(m % t, t);
+            u64 e0, e1;
+            pm_entry(mulmod(t % m, invmod(part(Qp, (int)i, m), m), m), m, b - 28, &e0, &e1);
+            for (u64 e : {e0, e1}) {
+                c->pm_dec.w.push_back((uint32_t)e);
+                c->pm_dec.w.push_back((uint32_t)(e >> 32));
+            }
+            c->pm_dec.q.push_back(m);
+            c->pm_dec.d.push_back((uint32_t)(((u64)1 << b) - m));
+            c->pm_dec.c.push_back((uint32_t)ci);
+            c->pm_dec.c2.push_back((uint32_t)mulmod(ci, ((u64)1 << hs) % t, t));
+        }
         // twist rows: t R N^-1 psi^-k of row 2 times the folded constant
         std::vector<u64> xtw((size_t)(L + K) * N * 2);
         for (uint32_t l = 0; l < L + K; ++l) {

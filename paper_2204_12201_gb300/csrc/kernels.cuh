@@ -24,6 +24,7 @@ int launch_modup(const bfhe_ctx* ctx, const u64* A, const u64* B, u64* X, int n,
 // the same for moduli 2^b - d with the guarded extension on (ext_pm.cu)
 int launch_modup_pm(const bfhe_ctx* ctx, const u64* A, const u64* B, u64* X, int n, int slots, cudaStream_t st);
 int launch_scale_pm(const bfhe_ctx* ctx, const u64* X, u64* C3, int n, cudaStream_t st, u64* tmp);
+int launch_dec_pm(const bfhe_ctx* ctx, const u64* V, const u64* ct, u64* M, int n, cudaStream_t st);
 int launch_tensor(const bfhe_ctx* ctx, u64* X, int n, int square, cudaStream_t st);
 // tmp: [n][3][K][N] words for the two-pass form (10 or more data primes), or null for one pass
 int launch_scale(const bfhe_ctx* ctx, const u64* X, u64* C3, int n, cudaStream_t st, u64* tmp = nullptr);

@@ -58,6 +58,8 @@ struct NttArgs {
     int n_inner;
     size_t in_os, in_is, in_ls, out_os, out_is, out_ls;
     const u64 *src0, *src1;   // limbs below src_limbs come from here (NttIO::src)
+    const u64* mul;           // the inverse's second factor (NttIO::mul)
+    size_t mul_os, mul_is;
     int src_limbs;
     int n_limbs;
     LimbMap map;
@@ -109,6 +111,7 @@ __device__ __forceinline__ ulonglong2 load_now(const ulonglong2* p) {
 struct LimbPtrs {
     const u64* in;   // limb start
     u64* out;        // limb start
+    const u64* mul;  // limb start
     int p;
 };
 
@@ -122,6 +125,7 @@ __device__ __forceinline__ LimbPtrs limb_ptrs(const NttArgs& a, int bx) {
                ? (inner < 2 ? a.src0 : a.src1) + ((size_t)(2 * outer + (inner & 1)) * a.src_limbs + limb) * a.N
                : a.in + outer * a.in_os + inner * a.in_is + limb * a.in_ls;
     r.out = a.out + outer * a.out_os + inner * a.out_is + limb * a.out_ls;
+    r.mul = FWD ? nullptr : a.mul + outer * a.mul_os + inner * a.mul_is + (size_t)limb * a.N;
     r.p = a.map(limb);
     return r;
 }
@@ -297,7 +301,8 @@ __device__ __forceinline__ void inv_stages(u64 (&x)[1 << LOG_E], int base, const
 
 // MODE 1: the block is the whole limb; MODE 2: half `half` of a limb of N = 2M words,
 // whose outermost stage pairs with the partner CTA of the cluster.
-// OUT 0: twisted, canonical; 2: not twisted (the consumer multiplies by the twist, folded into a product it makes
+// OUT 0: twisted, canonical; 1: the same, of the input times the words of mul (an evaluation-domain product that would
+// otherwise be a kernel and a round trip through memory of its own); 2: not twisted (the consumer multiplies by the twist, folded into a product it makes
 // anyway): from inputs below q, 15 stages leave words below 61q < 2^64, or signed words below 2^63 (PM).
 template <bool PM>
 __device__ __forceinline__ u64 twisted(u64 x, const ulonglong2& t, const Mod<PM>& m) {
@@ -307,8 +312,8 @@ __device__ __forceinline__ u64 twisted(u64 x, const ulonglong2& t, const Mod<PM>
 
 template <bool PM, int LOG_M, int LOG_E, int P, int MODE, int OUT>
 __device__ __forceinline__ void inv_pass(u64 (&x)[1 << LOG_E], u64* sm, int tid, const ulonglong2* itw,
-                                         const ulonglong2* twist, const Mod<PM>& m, const u64* in, u64* out, int half,
-                                         bool natural) {
+                                         const ulonglong2* twist, const Mod<PM>& m, const u64* in, u64* out, const u64* mul,
+                                         int half, bool natural) {
     constexpr int E = 1 << LOG_E;
     constexpr int M = 1 << LOG_M;
     constexpr int NPASS = (LOG_M + LOG_E - 1) / LOG_E;
@@ -336,6 +341,15 @@ __device__ __forceinline__ void inv_pass(u64 (&x)[1 << LOG_E], u64* sm, int tid,
                 x[2 * e + 1] = v.y;
             }
         }
+        if constexpr (OUT == 1) {
+            const ulonglong2* m2 = reinterpret_cast<const ulonglong2*>(mul + eval_pos(base));
+#pragma unroll
+            for (int e = 0; e < E / 2; ++e) {
+                const ulonglong2 v = m2[e * 32];
+                x[2 * e] = pm_mul_var(x[2 * e], v.x, m.q, m.b, m.d);
+                x[2 * e + 1] = pm_mul_var(x[2 * e + 1], v.y, m.q, m.b, m.d);
+            }
+        }
     } else {
 #pragma unroll
         for (int e = 0; e < E; ++e) x[e] = sm[pb + poff<W_LO>(e)];
@@ -347,7 +361,7 @@ __device__ __forceinline__ void inv_pass(u64 (&x)[1 << LOG_E], u64* sm, int tid,
         for (int e = 0; e < E; ++e) sm[pb + poff<W_LO>(e)] = x[e];
         constexpr int W_NEXT = LO + 2 * LOG_E <= LOG_M ? LO + LOG_E : LOG_M - LOG_E;
         exchange_sync<W_LO, W_NEXT>();
-        inv_pass<PM, LOG_M, LOG_E, P + 1, MODE, OUT>(x, sm, tid, itw, twist, m, in, out, half, natural);
+        inv_pass<PM, LOG_M, LOG_E, P + 1, MODE, OUT>(x, sm, tid, itw, twist, m, in, out, mul, half, natural);
     } else if constexpr (MODE == 2) {
         // outermost stage across the halves, pairs (j, j + M): the top bit of e is bit LOG_M - 1 of j, so
         // CTA 0 takes the pairs with j < M/2 and CTA 1 those with j >= M/2; each publishes the words of the
@@ -398,7 +412,7 @@ __device__ __forceinline__ void inv_pass(u64 (&x)[1 << LOG_E], u64* sm, int tid,
 }
 
 template <bool PM, int LOG_M, int LOG_E, int MODE, int OUT>
-__global__ void __launch_bounds__(1 << (LOG_M - LOG_E), (MODE == 2 && LOG_M < 14 && LOG_M - LOG_E <= 8 ? 2 : 1)) k_ntt_inv(NttArgs a) {
+__global__ void __launch_bounds__(1 << (LOG_M - LOG_E), (LOG_M < 14 && LOG_M - LOG_E <= 8 ? 2 : 1)) k_ntt_inv(NttArgs a) {
     extern __shared__ u64 sm[];
     const LimbPtrs lp = limb_ptrs<false>(a, blockIdx.x);
     const int half = blockIdx.y;
@@ -407,7 +421,8 @@ __global__ void __launch_bounds__(1 << (LOG_M - LOG_E), (MODE == 2 && LOG_M < 14
     const ulonglong2* twist = reinterpret_cast<const ulonglong2*>(a.tab.twist) + ((size_t)lp.p * 3 + (a.mont ? 1 : 0)) * a.N;
     u64 x[1 << LOG_E];
     inv_pass<PM, LOG_M, LOG_E, 0, MODE, OUT>(x, sm, threadIdx.x, itw, twist, m, lp.in + ((size_t)half << LOG_M),
-                                             lp.out + ((size_t)half << LOG_M), half, a.natural);
+                                             lp.out + ((size_t)half << LOG_M), lp.mul + ((size_t)half << LOG_M), half,
+                                             a.natural);
 }
 
 template <int LOG_M, int LOG_E>
@@ -489,6 +504,11 @@ int fwd_shape(const NttArgs& a, int blocks, cudaStream_t st, bool top) {
     return a.lazy ? run_fwd<PM, LM, LE, false, true>(a, blocks, st) : run_fwd<PM, LM, LE, false, false>(a, blocks, st);
 }
 
+template <int LM, int LE>
+int inv_mul_shape(const NttArgs& a, int blocks, cudaStream_t st, bool split) {
+    return split ? run_inv<true, LM, LE, 2, 1>(a, blocks, st) : run_inv<true, LM, LE, 1, 1>(a, blocks, st);
+}
+
 template <bool PM, int LM, int LE>
 int inv_shape(const NttArgs& a, int blocks, cudaStream_t st, bool split) {
     if (split)
@@ -508,13 +528,16 @@ int inv_shape(const NttArgs& a, int blocks, cudaStream_t st, bool split) {
     if (log_m == LM && log_e == LE) return fwd_shape<PM, LM, LE>(a, blocks, st, split);
 #define INV_CASE(LM, LE) \
     if (log_m == LM && log_e == LE) return inv_shape<PM, LM, LE>(a, blocks, st, split);
+#define INV_MUL_CASE(LM, LE) \
+    if (log_m == LM && log_e == LE) return inv_mul_shape<LM, LE>(a, blocks, st, split);
 
-// The shapes' kernels are compiled as four objects of this file (BFHE_NTT_PART: forward and inverse, without and
-// with pm), in parallel; part 0 also holds the host side.
+// The shapes' kernels are compiled as five objects of this file (BFHE_NTT_PART: forward and inverse, without and with
+// pm, and the inverse of a product), in parallel; part 0 also holds the host side.
 int ntt_fwd_any(const NttArgs& a, int log_m, int log_e, int blocks, bool split, cudaStream_t st);
 int ntt_fwd_any_pm(const NttArgs& a, int log_m, int log_e, int blocks, bool split, cudaStream_t st);
 int ntt_inv_any(const NttArgs& a, int log_m, int log_e, int blocks, bool split, cudaStream_t st);
 int ntt_inv_any_pm(const NttArgs& a, int log_m, int log_e, int blocks, bool split, cudaStream_t st);
+int ntt_inv_mul_any_pm(const NttArgs& a, int log_m, int log_e, int blocks, bool split, cudaStream_t st);
 
 #if BFHE_NTT_PART == 0
 int ntt_fwd_any(const NttArgs& a, int log_m, int log_e, int blocks, bool split, cudaStream_t st) {
@@ -534,10 +557,15 @@ int ntt_inv_any(const NttArgs& a, int log_m, int log_e, int blocks, bool split, 
     NTT_SHAPES(INV_CASE)
     return set_error(BFHE_EINVAL, "no NTT configuration for this ring degree");
 }
-#else
+#elif BFHE_NTT_PART == 3
 int ntt_inv_any_pm(const NttArgs& a, int log_m, int log_e, int blocks, bool split, cudaStream_t st) {
     constexpr bool PM = true;
     NTT_SHAPES(INV_CASE)
+    return set_error(BFHE_EINVAL, "no NTT configuration for this ring degree");
+}
+#elif BFHE_NTT_PART == 4
+int ntt_inv_mul_any_pm(const NttArgs& a, int log_m, int log_e, int blocks, bool split, cudaStream_t st) {
+    NTT_SHAPES(INV_MUL_CASE)
     return set_error(BFHE_EINVAL, "no NTT configuration for this ring degree");
 }
 #endif
@@ -564,6 +592,9 @@ NttArgs make_args(const bfhe_ctx* ctx, const NttIO& io, int n_limbs, LimbMap map
     a.src0 = io.src[0];
     a.src1 = io.src[1];
     a.src_limbs = io.src_limbs;
+    a.mul = io.mul;
+    a.mul_os = io.mul_os;
+    a.mul_is = io.mul_is;
     a.natural = io.natural;
     a.bits = (int)ctx->prime_bits;
     a.mont = mont;
@@ -581,11 +612,13 @@ int env_int(const char* name) {
 
 // Block size and registers per thread.  Defaults (measured on GB300 inside the multiply, pm products, us per
 // launch class, forward / inverse): N <= 4096 in one block of 16 words per thread (64 pairs at N = 4096, L = 2: 52 / 41;
-// 32 words 59 / 88, halves 54 / 53).  N = 8192 in one block of 32 words (64 pairs, L = 4: 201 / 147; 16 words 231 /
-// 152).  N = 16384 in one block of 32 words (64 pairs, L = 8: 1022 / 516; halves 1031 / 560).  N = 32768 as two
-// 16384-word halves, 32 words (8 pairs, L = 16: 889 / 348; 16 words 950 / 475).  A launch at N = 16384 whose halves
-// fit the 152 SMs at one CTA each takes halves at 16 words, twice the threads on each limb (one pair, L = 8: 33 / 33
-// against 44 / 42).  bfhe_ntt_config (the autotuner) or BFHE_NTT_LOG_M / BFHE_NTT_LOG_E override the defaults.
+// 32 words 61 / 87, halves 54 / 53).  N = 8192 in one block of 32 words, two blocks per SM (64 pairs, L = 4: 196 / 137;
+// 16 words 233 / 151).  N = 16384 in one block of 32 words (64 pairs, L = 8: 1017 / 515; halves 1029 / 559).  N = 32768
+// as two 16384-word halves, 32 words (8 pairs, L = 16: 887 / 347; 16 words 949 / 471).  A launch whose halves fit the 152
+// SMs at one CTA each takes halves at 16 words, which puts twice the threads on each limb: at N = 16384 (72 limbs: 14 / 15
+// against 19 / 19) and for the forward at N = 8192 (8.3 against 12.5); the inverse there takes one block of 16 words
+// (up to 152 limbs: 10.4 to 11.7 against 12.4; halves 10.3).  bfhe_ntt_config (the autotuner) or BFHE_NTT_LOG_M /
+// BFHE_NTT_LOG_E override the defaults.
 int g_cfg[16][2][2] = {};   // [logN][inverse] -> (log_m, log_e), 0 = default
 
 int ntt_config(int logN, int inverse, size_t limbs, int* log_m, int* log_e) {
@@ -593,10 +626,11 @@ int ntt_config(int logN, int inverse, size_t limbs, int* log_m, int* log_e) {
     static const int env_e = env_int("BFHE_NTT_LOG_E");
     int m = logN <= 14 ? logN : logN - 1;
     int e = logN >= 13 ? 5 : 4;
-    if (logN == 14 && 2 * limbs <= 152) {
-        m = 13;
+    if ((logN == 14 || (logN == 13 && !inverse)) && 2 * limbs <= 152) {
+        m = logN - 1;
         e = 4;
     }
+    if (logN == 13 && inverse && limbs <= 152) e = 4;
     if (env_m >= logN - 1 && env_m <= logN && env_m >= 10 && env_m <= 14) m = env_m;
     if (env_e >= 3 && env_e <= 5) e = env_e;
     if (logN >= 0 && logN < 16 && g_cfg[logN][inverse ? 1 : 0][0]) {
@@ -656,6 +690,10 @@ int launch_ntt_inv(const bfhe_ctx* ctx, NttIO io, int n_polys, int n_limbs, Limb
     if (subs != 1 && subs != 2) return set_error(BFHE_EINVAL, "unsupported ring degree");
     if (lazy_out != 0 && lazy_out != 2) return set_error(BFHE_EINVAL, "bad inverse output form");
     const bool pm = ctx->pm && map(0) != (int)ctx->nP - 1;
+    if (io.mul) {
+        if (!pm || lazy_out) return set_error(BFHE_EINVAL, "the inverse of a product needs moduli 2^b - d");
+        return ntt_inv_mul_any_pm(a, log_m, log_e, blocks, subs == 2, st);
+    }
     return pm ? ntt_inv_any_pm(a, log_m, log_e, blocks, subs == 2, st)
               : ntt_inv_any(a, log_m, log_e, blocks, subs == 2, st);
 }

@@ -70,3 +70,36 @@ def test_extension_forms_agree(bits, L, alpha):
         assert torch.equal(x, y)
     ctx.check()
     ctx.close()
+
+
+@pytest.mark.parametrize("bits,t", [(45, 65537), (50, 65537), (55, 65537), (50, 12289), (50, 2)])
+@pytest.mark.parametrize("N,L", [(1024, 1), (1024, 8), (2048, 16)])
+def test_decryption_forms_agree(bits, t, N, L):
+    """Decryption's last step as folded sums and by mixed radix, on uniform residues and on words whose plaintext
+    lies at a rounding boundary; the plain product (inverse of an evaluation-domain product) against slot products."""
+    need_gpu()
+    import __graft_entry__
+    __graft_entry__.build()
+    from paper_2204_12201_gb300 import bfhe
+    ctx = bfhe.Context(N=N, L=L, alpha=1, t=t, prime_bits=bits)
+    ctx.keygen(4)
+    Q = 1
+    for p in ctx.primes[:L]:
+        Q *= p
+    g = torch.Generator(device="cuda").manual_seed(bits + L)
+    q = torch.tensor(ctx.primes[:L], device="cuda").view(1, 1, L, 1)
+    ct = torch.randint(0, 1 << 62, (3, 2, L, N), device="cuda", generator=g) % q
+    ct[1:, 1] = 0   # c1 = 0: c0 alone is decrypted, k/t Q + a half either side
+    for m, x in enumerate([0, 1, Q - 1, Q // (2 * t), Q // (2 * t) + 1, Q // 2, Q // 2 + 1, 3 * Q // (2 * t)]):
+        ct[1, 0, :, m::8] = torch.tensor([x % p for p in ctx.primes[:L]], device="cuda").view(L, 1)
+    new = ctx.decrypt_poly(ct)
+    assert ctx.lib.bfhe_set_fast_extension(ctx.h, 0) == 0
+    assert torch.equal(new, ctx.decrypt_poly(ct))
+    assert ctx.lib.bfhe_set_fast_extension(ctx.h, 1) in (0, -1)
+    assert bool((new >= 0).all()) and bool((new < t).all())
+    if t != 2 and L == 8:
+        y = torch.from_numpy(inputs.slots(3, 2, N, hi=t)).cuda()
+        w = torch.from_numpy(inputs.slots(5, 2, N, hi=t)).cuda()
+        assert torch.equal(ctx.decrypt(ctx.mul_plain(ctx.encrypt(y, 1), w)), y * w % t)
+    ctx.check()
+    ctx.close()

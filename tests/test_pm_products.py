@@ -203,3 +203,24 @@ def test_warp_exchanges_stay_inside_the_warp(m, e):
             if a <= 5 and b <= 5:
                 for warp in range((1 << (m - e)) // 32):
                     assert words(a, warp) == words(b, warp)
+
+
+@pytest.mark.parametrize("bits", [45, 50, 55])
+def test_product_of_two_run_time_factors(bits):
+    """pm_mul_var: the 128-bit product of factors below 2^(bits+1) folded to a canonical residue."""
+    rng = random.Random(bits)
+    for N, L in [(1024, 1), (32768, 16)]:
+        q = Params(N=N, L=L, alpha=1, prime_bits=bits).b[-1]
+        d, s, M = (1 << bits) - q, bits - 32, (1 << 32) - 1
+        top_v = (1 << (bits + 1)) - 1
+        for a, b in [(0, 0), (top_v, top_v), (q - 1, q - 1), (top_v, 1)] + [(rng.randrange(top_v), rng.randrange(top_v)) for _ in range(50)]:
+            a0, a1, b0, b1 = a & M, a >> 32, b & M, b >> 32
+            lo = a0 * b0
+            m = a1 * b0 + (lo >> 32) + a0 * b1
+            top = a1 * b1 + (m >> 32)
+            assert m < 1 << 64 and top < 1 << 64
+            h0, h1 = ((m & M) | (top & M) << 32) >> s & M, u32(top >> s)
+            g = h1 * d
+            assert g < 1 << 64
+            r = ((m & ((1 << s) - 1)) << 32 | lo & M) + ((g & ((1 << s) - 1)) << 32) + h0 * d + u32(g >> s) * d
+            assert r < 1 << 63 and (r - a * b) % q == 0
