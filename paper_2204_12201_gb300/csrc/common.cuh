@@ -365,6 +365,40 @@ int cuda_check(cudaError_t e, const char* where);
         if (_e != cudaSuccess) return cuda_check(_e, where);     \
     } while (0)
 
+// Every kernel of the library starts with pdl_begin and is launched with launch_kernel: the launch of a kernel, its
+// blocks' arrival and its reads of constant tables overlap the tail of the one before it on the stream (programmatic
+// dependent launch), and nothing that an earlier kernel writes, or still reads, is touched before pdl_wait returns, which
+// is when that kernel has completed.  Measured on GB300, calls one after another: a multiply of one pair at N = 16384,
+// L = 8 102 -> 81 us, of 64 pairs at N = 4096, L = 2 159 -> 145 us, of 64 at N = 16384 2510 -> 2491 us; one XOR gate at
+// N = 4096 53 -> 37 us.  Inside a CUDA graph the plain dependency is the cheaper one (16-bit comparator at N = 4096
+// replayed: 263 us, with programmatic edges 286), so a launch on a capturing stream leaves the attribute out.
+__device__ __forceinline__ void pdl_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_begin() {
+    pdl_next();
+    pdl_wait();
+}
+template <class... P, class... A>
+cudaError_t launch_kernel(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, int cluster_y, A&&... a) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at[2];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    const bool plain = cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone;
+    at[0].val.programmaticStreamSerializationAllowed = plain ? 0 : 1;
+    at[1].id = cudaLaunchAttributeClusterDimension;
+    at[1].val.clusterDim.x = 1;
+    at[1].val.clusterDim.y = cluster_y;
+    at[1].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = cluster_y > 1 ? 2 : 1;
+    return cudaLaunchKernelEx(&cfg, kern, static_cast<P>(a)...);
+}
+
 // scratch arena: returns a pointer to at least `bytes` bytes (grows, syncing the device)
 int ctx_scratch(bfhe_ctx* ctx, size_t bytes, void** out);
 // bytes of scratch one mul_relin of n ciphertexts needs

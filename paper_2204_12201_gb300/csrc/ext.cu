@@ -122,6 +122,7 @@ __device__ __forceinline__ u64 fast_eval3(const uint32_t (&y0)[NS], const uint32
 template <int NS, bool FAST>
 __global__ void __launch_bounds__(256, NS <= 8 ? 4 : 2) k_modup(const u64* A, const u64* B, u64* X, int n, int slots, int K, ExtDesc ext, int N,
                         uint32_t* flags, FastTab<FAST ? NS : 1, FAST ? NS + 1 : 1> ft) {
+    pdl_begin();
     const size_t total = (size_t)n * slots * N;
     const int LK = NS + K;
     for (size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
@@ -162,6 +163,7 @@ template <int NS, int KS, bool FAST>
 __global__ void __launch_bounds__(256, 2) k_scale(const u64* X, u64* C3, int n, ExtDesc eQB, ExtDesc eBQ, const u64* twist, int nP,
                         const u64* Qinv_b, const u64* bq, int N, int bits, FastTab<FAST ? NS : 1, FAST ? KS : 1> fq,
                         FastTab<FAST ? KS : 1, FAST ? NS : 1> fb) {
+    pdl_begin();
     const size_t total = (size_t)n * 3 * N;
     constexpr int LK = NS + KS;
     for (size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
@@ -226,6 +228,7 @@ __global__ void __launch_bounds__(256, 2) k_scale(const u64* X, u64* C3, int n, 
 template <int NS, int KS>
 __global__ void __launch_bounds__(256, 2) k_scale_a(const u64* X, u64* Yt, int n, ExtDesc eQB, const u64* twist, int nP,
                                                     const u64* Qinv_b, const u64* bq, int N, int bits, FastTab<NS, KS> fq) {
+    pdl_begin();
     const size_t total = (size_t)n * 3 * N;
     constexpr int LK = NS + KS;
     for (size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
@@ -282,6 +285,7 @@ __global__ void __launch_bounds__(256, 2) k_scale_a(const u64* X, u64* Yt, int n
 template <int NS, int KS>
 __global__ void __launch_bounds__(256, 2) k_scale_b(const u64* Yt, u64* C3, int n, ExtDesc eBQ, int N,
                                                     FastTab<KS, NS> fb) {
+    pdl_begin();
     const size_t total = (size_t)n * 3 * N;
     for (size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
          idx += (size_t)gridDim.x * blockDim.x) {
@@ -311,6 +315,7 @@ __global__ void __launch_bounds__(256, 2) k_scale_b(const u64* Yt, u64* C3, int 
 template <int NA>
 __global__ void k_moddown(const u64* W, const u64* C3, u64* out, int n, int L, ExtDesc ePQ, const u64* Pinv,
                           const u64* qtab, const u64* twist, int N, int bits) {
+    pdl_begin();
     // two consecutive coefficients per thread (N is even, every limb starts 16-byte aligned): 16-byte accesses
     const size_t half = (size_t)N >> 1;
     const size_t total = (size_t)n * 2 * half;
@@ -353,6 +358,7 @@ __global__ void k_moddown(const u64* W, const u64* C3, u64* out, int n, int L, E
 template <int NS>
 __global__ void k_dec_finish(const u64* V, const u64* ct, u64* M, int n, ExtDesc eQt, const u64* tmod, int nP,
                              u64 Qinv_t, int N, uint32_t* flags) {
+    pdl_begin();
     const size_t total = (size_t)n * N;
     for (size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
          idx += (size_t)gridDim.x * blockDim.x) {
@@ -381,6 +387,7 @@ __global__ void k_dec_finish(const u64* V, const u64* ct, u64* M, int n, ExtDesc
 // instance per size; the guarded fast extension is not offered there.
 __global__ void k_modup_n(const u64* A, const u64* B, u64* X, int n, int slots, int K, ExtDesc ext, int N,
                           uint32_t* flags) {
+    pdl_begin();
     const int ns = ext.n_src;
     const size_t total = (size_t)n * slots * N;
     const int LK = ns + K;
@@ -406,6 +413,7 @@ __global__ void k_modup_n(const u64* A, const u64* B, u64* X, int n, int slots, 
 
 __global__ void k_scale_n(const u64* X, u64* C3, int n, ExtDesc eQB, ExtDesc eBQ, const u64* twist, int nP,
                           const u64* Qinv_b, const u64* bq, int N, int bits) {
+    pdl_begin();
     const int ns = eQB.n_src, ks = eBQ.n_src, LK = ns + ks;
     const size_t total = (size_t)n * 3 * N;
     for (size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
@@ -437,6 +445,7 @@ __global__ void k_scale_n(const u64* X, u64* C3, int n, ExtDesc eQB, ExtDesc eBQ
 
 __global__ void k_dec_finish_n(const u64* V, const u64* ct, u64* M, int n, ExtDesc eQt, const u64* tmod, int nP,
                                u64 Qinv_t, int N, uint32_t* flags) {
+    pdl_begin();
     const int ns = eQt.n_src;
     const size_t total = (size_t)n * N;
     for (size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total;

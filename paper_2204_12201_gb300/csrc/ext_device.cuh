@@ -135,7 +135,7 @@ __device__ u64 ext_eval_n(const u64* v, bool neg, const ExtDesc& d, int j, int n
 #define LAUNCH(kern, work, ...)                                                   \
     do {                                                                          \
         auto* _kfn = kern;                                                        \
-        _kfn<<<grid_for(work), TPB, 0, st>>>(__VA_ARGS__);                       \
+        BFHE_CUDA(launch_kernel(_kfn, dim3(grid_for(work)), dim3(TPB), 0, st, 1, __VA_ARGS__)); \
         BFHE_LAUNCH_CHECK(#kern);                                                \
     } while (0)
 

@@ -153,6 +153,7 @@ __global__ void __launch_bounds__(256, NS <= 8 ? 4 : 2)
     k_modup_pm(const u64* __restrict__ A, const u64* __restrict__ B, u64* __restrict__ X, int n, int slots, int logN, int b,
                ExtDesc ext, uint32_t* flags, const __grid_constant__ PrepTab<NS> p,
                const __grid_constant__ SumTab<NS, NS + 1> t) {
+    pdl_begin();
     constexpr int KS = NS + 1, LK = NS + KS;
     const int N = 1 << logN, k = b - 28, hs = (b + 2) >> 1;
     const size_t total = (size_t)n * slots << logN;
@@ -253,6 +254,7 @@ __global__ void __launch_bounds__(256, 2)
     k_scale_pm(const u64* __restrict__ X, u64* __restrict__ C3, int n, int logN, int b, const ulonglong2* __restrict__ xtw,
                const __grid_constant__ SumTab<NS, NS + 1> tq, const __grid_constant__ SumTab<NS + 1, NS> tb,
                const __grid_constant__ ExactScale ex) {
+    pdl_begin();
     constexpr int KS = NS + 1, LK = NS + KS;
     const int N = 1 << logN, hs = (b + 2) >> 1;
     const size_t total = (size_t)n * 3 << logN;
@@ -295,6 +297,7 @@ template <int NS>
 __global__ void __launch_bounds__(256, 2)
     k_scale_pm_a(const u64* __restrict__ X, u64* __restrict__ Z, int n, int logN, int b, const ulonglong2* __restrict__ xtw,
                  const __grid_constant__ SumTab<NS, NS + 1> tq, const __grid_constant__ SumTab<NS + 1, NS> tb) {
+    pdl_begin();
     constexpr int KS = NS + 1, LK = NS + KS;
     const int N = 1 << logN;
     const size_t total = (size_t)n * 3 << logN;
@@ -325,6 +328,7 @@ template <int NS>
 __global__ void __launch_bounds__(256, 2)
     k_scale_pm_b(const u64* __restrict__ X, const u64* __restrict__ Z, u64* __restrict__ C3, int n, int logN, int b,
                  const __grid_constant__ SumTab<NS + 1, NS> tb, const __grid_constant__ ExactScale ex) {
+    pdl_begin();
     constexpr int KS = NS + 1, LK = NS + KS;
     const int N = 1 << logN, hs = (b + 2) >> 1;
     const size_t total = (size_t)n * 3 << logN;
@@ -376,6 +380,7 @@ template <int NS>
 __global__ void __launch_bounds__(256, 4)
     k_dec_pm(const u64* __restrict__ V, const u64* __restrict__ ct, u64* __restrict__ M, int n, int logN, int b, ExtDesc ext,
              const u64* tmod, int nP, uint32_t* flags, const __grid_constant__ DecTab<NS> p) {
+    pdl_begin();
     const int k = b - 28, hs = (b + 2) >> 1;
     const size_t total = (size_t)n << logN;
     for (size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total;

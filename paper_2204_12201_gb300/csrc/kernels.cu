@@ -43,6 +43,7 @@ __device__ __forceinline__ void philox4x64(u64 c[4], u64 k0, u64 k1) {
 
 __global__ void k_sample_uniform(u64* out, int n_polys, int n_limbs, LimbMap map, PrimeTab tab, const u64* R2,
                                  u64 seed, u64 purpose, u64 poly_base, int N) {
+    pdl_begin();
     const size_t half = (size_t)N >> 1;
     const size_t total = (size_t)n_polys * n_limbs * half;
     for (size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
@@ -65,6 +66,7 @@ __global__ void k_sample_uniform(u64* out, int n_polys, int n_limbs, LimbMap map
 }
 
 __global__ void k_sample_small(i64* out, int n_polys, u64 seed, u64 purpose, u64 poly_base, int cbd, int N) {
+    pdl_begin();
     const size_t quarter = (size_t)N >> 2;
     const size_t total = (size_t)n_polys * quarter;
     for (size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
@@ -88,6 +90,7 @@ __global__ void k_sample_small(i64* out, int n_polys, u64 seed, u64 purpose, u64
 }
 
 __global__ void k_spread(const i64* in, u64* out, int n_polys, int n_limbs, LimbMap map, PrimeTab tab, int N) {
+    pdl_begin();
     const size_t total = (size_t)n_polys * n_limbs * N;
     for (size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
          idx += (size_t)gridDim.x * blockDim.x) {
@@ -103,6 +106,7 @@ __global__ void k_spread(const i64* in, u64* out, int n_polys, int n_limbs, Limb
 // ---------------------------------------------------------------- pointwise (NTT domain)
 __global__ void k_pointwise(const u64* A, const u64* B, u64* out, int n, int polys, int n_limbs, LimbMap map,
                             PrimeTab tab, PwStrides s, int N) {
+    pdl_begin();
     const size_t total = (size_t)n * polys * n_limbs * N;
     for (size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
          idx += (size_t)gridDim.x * blockDim.x) {
@@ -134,6 +138,7 @@ __device__ __forceinline__ void tensor_word(u64 a0, u64 a1, u64 b0, u64 b1, u64 
 }
 
 __global__ void k_tensor(u64* X, int n, int LK, LimbMap map, PrimeTab tab, int N) {
+    pdl_begin();
     const size_t plane = (size_t)LK * N, half = plane / 2;
     const size_t total = (size_t)n * half;
     for (size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
@@ -155,6 +160,7 @@ __global__ void k_tensor(u64* X, int n, int LK, LimbMap map, PrimeTab tab, int N
 
 // squaring: X[c][0..1] = (a0, a1) -> X[c][0..2] = (a0^2, 2 a0 a1, a1^2), same sums as the general tensor
 __global__ void k_tensor_sq(u64* X, int n, int LK, LimbMap map, PrimeTab tab, int N) {
+    pdl_begin();
     const size_t plane = (size_t)LK * N, half = plane / 2;
     const size_t total = (size_t)n * half;
     for (size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
@@ -198,6 +204,7 @@ __device__ __forceinline__ void join28(u64 sl, u64 sm, u64 sh, u64& hi, u64& lo)
 template <int L, bool SPLIT>
 __global__ void __launch_bounds__(256, 2) k_inner(const u64* Dg, const u64* rlk, u64* W, int n, int QP,
                                                               int cpg, PrimeTab tab, int N) {
+    pdl_begin();
     static_assert(!SPLIT || L <= 16, "the split sums are bounded for at most 16 terms");
     constexpr int D = L <= 8 ? 2 : 0;
     constexpr uint32_t M28 = (1u << 28) - 1;
@@ -275,6 +282,7 @@ __global__ void __launch_bounds__(256, 2) k_inner(const u64* Dg, const u64* rlk,
 // the same inner product for 17 or more data primes (insecure test-only parameter sets): sizes at run time,
 // one thread per (ciphertext, word), the key re-read per ciphertext
 __global__ void k_inner_n(const u64* Dg, const u64* rlk, u64* W, int n, int QP, int L, PrimeTab tab, int N) {
+    pdl_begin();
     const size_t plane = (size_t)QP * N;
     const size_t total = plane * n;
     for (size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
@@ -299,6 +307,7 @@ __global__ void k_inner_n(const u64* Dg, const u64* rlk, u64* W, int n, int QP, 
 // ---------------------------------------------------------------- encode/decode, encrypt, keygen
 __global__ void k_permute(const u64* in, u64* out, const uint32_t* brv, int n, int scatter, int N, u64 t,
                           uint32_t* flags) {
+    pdl_begin();
     const size_t total = (size_t)n * N;
     for (size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
          idx += (size_t)gridDim.x * blockDim.x) {
@@ -317,6 +326,7 @@ __global__ void k_permute(const u64* in, u64* out, const uint32_t* brv, int n, i
 // out = -(as + e) [+ [P]_{q_j} s2 on limb j of poly j when gadget]
 __global__ void k_neg_add_small(const u64* as, const i64* e, u64* out, int n_polys, int n_limbs, LimbMap map,
                                 PrimeTab tab, const u64* s2, int gadget, const u64* Pq, int L, int N) {
+    pdl_begin();
     const size_t total = (size_t)n_polys * n_limbs * N;
     for (size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
          idx += (size_t)gridDim.x * blockDim.x) {
@@ -421,6 +431,7 @@ __device__ __forceinline__ Words<W> lin_words(int cc, int cx, int cy, int cz, in
 template <int W>
 __global__ void __launch_bounds__(256) k_lincomb(u64* out, const u64* x, const u64* y, const u64* z, const u64* p, LinCoef cf,
                                                  u64 cval, int L, const u64* qtab, const u64* delta, int logN) {
+    pdl_begin();
     const Row<W> r(logN);
     const uint32_t h = r.row / (uint32_t)L;
     const int i = (int)(r.row - h * L);
@@ -434,6 +445,7 @@ struct ScalarPairs {
 
 template <int W>
 __global__ void __launch_bounds__(256) k_mul_scalar(const u64* a, u64* out, ScalarPairs sp, int L, const u64* qtab, int logN) {
+    pdl_begin();
     const Row<W> r(logN);
     const int i = (int)(r.row % (uint32_t)L);
     const u64 q = qtab[i], w = sp.w[i], ws = sp.ws[i];
@@ -447,6 +459,7 @@ __global__ void __launch_bounds__(256) k_mul_scalar(const u64* a, u64* out, Scal
 template <int W>
 __global__ void __launch_bounds__(256) k_horner(const u64* bits, uint32_t s, u64* out, size_t words, int L, const u64* qtab,
                                                 int logN) {
+    pdl_begin();
     const Row<W> r(logN);
     const u64 q = qtab[r.row % (uint32_t)L];
     const u64* p = bits + (size_t)(s - 1) * words + r.off;
@@ -465,6 +478,7 @@ __global__ void __launch_bounds__(256) k_horner(const u64* bits, uint32_t s, u64
 template <int W>
 __global__ void __launch_bounds__(256) k_gather_ops(u64* A, u64* B, const u64* wires, uint32_t rows, const int32_t* table, int L,
                                                     const u64* qtab, int logN) {
+    pdl_begin();
     const Row<W> r(logN);
     const uint32_t g = r.row / rows, lr = r.row - g * rows;
     const size_t ctw = (size_t)rows << logN, o = ((size_t)lr << logN) + r.k;
@@ -484,6 +498,7 @@ __global__ void __launch_bounds__(256) k_gather_ops(u64* A, u64* B, const u64* w
 template <int W>
 __global__ void __launch_bounds__(256) k_gate_epilogue(u64* wires, uint32_t rows, const int32_t* table, int n_mul, const u64* prod,
                                                        int L, const u64* qtab, const u64* delta, int logN) {
+    pdl_begin();
     const Row<W> r(logN);
     const uint32_t g = r.row / rows, lr = r.row - g * rows;
     const size_t ctw = (size_t)rows << logN, o = ((size_t)lr << logN) + r.k;
@@ -523,6 +538,7 @@ __global__ void __launch_bounds__(256) k_gate_epilogue(u64* wires, uint32_t rows
 template <int W>
 __global__ void __launch_bounds__(256) k_enc_finish(u64* ct, const u64* M, const i64* e1, const i64* e2, int L, const u64* qtab,
                                                     const u64* delta, int logN, u64 t, uint32_t* flags) {
+    pdl_begin();
     const Row<W> r(logN);
     const uint32_t c = r.row / (uint32_t)L, i = r.row - c * L;
     const u64 q = qtab[i];
@@ -546,6 +562,7 @@ __global__ void __launch_bounds__(256) k_enc_finish(u64* ct, const u64* M, const
 
 // integer-pipe probe: 8 independent lazy Shoup chains per thread
 __global__ void k_probe_modmul(u64* out, uint32_t iters, u64 q, u64 w, u64 ws) {
+    pdl_begin();
     u64 x[8];
 #pragma unroll
     for (int i = 0; i < 8; ++i) x[i] = (u64)threadIdx.x * 977u + (u64)blockIdx.x * 131u + (u64)i;
@@ -563,6 +580,7 @@ __global__ void k_probe_modmul(u64* out, uint32_t iters, u64 q, u64 w, u64 ws) {
 template <int W>
 __global__ void __launch_bounds__(256) k_trivial_bits(u64* out, u64 c_base, const u64* cbp, uint32_t C, uint32_t n, int L,
                                                       const u64* delta, int logN) {
+    pdl_begin();
     const Row<W> r(logN);
     if (cbp) c_base = *cbp;
     const uint32_t h = r.row / (uint32_t)L, i = r.row - h * L;   // h: (bit, c, n, component)
@@ -576,6 +594,7 @@ __global__ void __launch_bounds__(256) k_trivial_bits(u64* out, u64 c_base, cons
 template <int W>
 __global__ void __launch_bounds__(256) k_accumulate(u64* bits, const u64* src, uint32_t rows, u64 c_base, const u64* cbp, int C,
                                                     int select, int L, const u64* qtab, int logN) {
+    pdl_begin();
     const Row<W> r(logN);
     if (cbp) c_base = *cbp;
     const uint32_t kbit = r.row / rows, lr = r.row - kbit * rows;
@@ -597,6 +616,7 @@ __global__ void __launch_bounds__(256) k_accumulate(u64* bits, const u64* src, u
 template <int W>
 __global__ void __launch_bounds__(256) k_sub_const_chains(const u64* x, u64* out, uint32_t rows, u64 c_base, const u64* cbp, int L,
                                                           const u64* qtab, const u64* delta, u64 t, int logN) {
+    pdl_begin();
     const Row<W> r(logN);
     if (cbp) c_base = *cbp;
     const uint32_t c = r.row / rows, lr = r.row - c * rows;
@@ -610,7 +630,7 @@ __global__ void __launch_bounds__(256) k_sub_const_chains(const u64* x, u64* out
 }
 
 // one device word (the candidate base read by a replayed mod_to_bits tile)
-__global__ void k_set_word(u64* w, u64 v) { *w = v; }
+__global__ void k_set_word(u64* w, u64 v) { pdl_begin(); *w = v; }
 
 }  // namespace
 
@@ -618,7 +638,7 @@ __global__ void k_set_word(u64* w, u64 v) { *w = v; }
 #define LAUNCH(kern, work, ...)                                                   \
     do {                                                                          \
         auto* _kfn = kern;                                                        \
-        _kfn<<<grid_for(work), TPB, 0, st>>>(__VA_ARGS__);                       \
+        BFHE_CUDA(launch_kernel(_kfn, dim3(grid_for(work)), dim3(TPB), 0, st, 1, __VA_ARGS__)); \
         BFHE_LAUNCH_CHECK(#kern);                                                \
     } while (0)
 
@@ -713,8 +733,10 @@ int launch_permute(const bfhe_ctx* ctx, const u64* in, u64* out, int n, int scat
 #define LAUNCH_ROWS(kern, wide, rows, ...)                                                                     \
     do {                                                                                                       \
         const size_t _rows = (rows);                                                                           \
-        if (wide) kern<2><<<(unsigned)(_rows << (ctx->logN - 9)), TPB, 0, st>>>(__VA_ARGS__);                  \
-        else kern<1><<<(unsigned)(_rows << (ctx->logN - 8)), TPB, 0, st>>>(__VA_ARGS__);                       \
+        if (wide)                                                                                              \
+            BFHE_CUDA(launch_kernel(kern<2>, dim3((unsigned)(_rows << (ctx->logN - 9))), dim3(TPB), 0, st, 1, __VA_ARGS__)); \
+        else                                                                                                   \
+            BFHE_CUDA(launch_kernel(kern<1>, dim3((unsigned)(_rows << (ctx->logN - 8))), dim3(TPB), 0, st, 1, __VA_ARGS__)); \
         BFHE_LAUNCH_CHECK(#kern);                                                                              \
     } while (0)
 
@@ -799,13 +821,13 @@ int launch_sub_const_chains(const bfhe_ctx* ctx, const u64* x, u64* out, u64 c_b
 }
 
 int launch_set_word(u64* w, u64 v, cudaStream_t st) {
-    k_set_word<<<1, 1, 0, st>>>(w, v);
+    BFHE_CUDA(launch_kernel(k_set_word, dim3(1), dim3(1), 0, st, 1, w, v));
     BFHE_LAUNCH_CHECK("k_set_word");
     return BFHE_OK;
 }
 
 int launch_probe_modmul(u64* out, int blocks, int threads, uint32_t iters, u64 q, u64 w, u64 ws, cudaStream_t st) {
-    k_probe_modmul<<<blocks, threads, 0, st>>>(out, iters, q, w, ws);
+    BFHE_CUDA(launch_kernel(k_probe_modmul, dim3(blocks), dim3(threads), 0, st, 1, out, iters, q, w, ws));
     BFHE_LAUNCH_CHECK("k_probe_modmul");
     return BFHE_OK;
 }

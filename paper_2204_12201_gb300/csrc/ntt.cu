@@ -263,6 +263,7 @@ __global__ void __launch_bounds__(1 << (LOG_M - LOG_E), (LOG_M < 14 && LOG_M - L
     const u64 jglob = (u64)a.N + ((u64)half << LOG_M);
     const u64* in = TOP ? lp.in : lp.in + ((size_t)half << LOG_M);
     u64 x[1 << LOG_E];
+    pdl_begin();
     fwd_pass<PM, LOG_M, LOG_E, 0, TOP, LAZY>(x, sm, threadIdx.x, jglob, tw, twl, m, mu, in,
                                              lp.out + ((size_t)half << LOG_M), half, a.natural);
 }
@@ -420,6 +421,7 @@ __global__ void __launch_bounds__(1 << (LOG_M - LOG_E), (LOG_M < 14 && LOG_M - L
     const ulonglong2* itw = reinterpret_cast<const ulonglong2*>(a.tab.itw) + (size_t)lp.p * a.N;
     const ulonglong2* twist = reinterpret_cast<const ulonglong2*>(a.tab.twist) + ((size_t)lp.p * 3 + (a.mont ? 1 : 0)) * a.N;
     u64 x[1 << LOG_E];
+    pdl_begin();
     inv_pass<PM, LOG_M, LOG_E, 0, MODE, OUT>(x, sm, threadIdx.x, itw, twist, m, lp.in + ((size_t)half << LOG_M),
                                              lp.out + ((size_t)half << LOG_M), lp.mul + ((size_t)half << LOG_M), half,
                                              a.natural);
@@ -441,25 +443,8 @@ int run_fwd(const NttArgs& a, int blocks, cudaStream_t st) {
                                        (int)smem));
         attr.fetch_or(1ull << dev);
     }
-    if (TOP) {
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3(blocks, 2, 1);
-        cfg.blockDim = dim3(T, 1, 1);
-        cfg.dynamicSmemBytes = smem;
-        cfg.stream = st;
-        cudaLaunchAttribute at[1];
-        at[0].id = cudaLaunchAttributeClusterDimension;
-        at[0].val.clusterDim.x = 1;
-        at[0].val.clusterDim.y = 2;
-        at[0].val.clusterDim.z = 1;
-        cfg.attrs = at;
-        cfg.numAttrs = 1;
-        BFHE_CUDA(cudaLaunchKernelEx(&cfg, k_ntt_fwd<PM, LOG_M, LOG_E, TOP, LAZY>, a));
-        BFHE_LAUNCH_CHECK("k_ntt_fwd (cluster)");
-    } else {
-        k_ntt_fwd<PM, LOG_M, LOG_E, TOP, LAZY><<<dim3(blocks, 1), T, smem, st>>>(a);
-        BFHE_LAUNCH_CHECK("k_ntt_fwd");
-    }
+    BFHE_CUDA(launch_kernel(k_ntt_fwd<PM, LOG_M, LOG_E, TOP, LAZY>, dim3(blocks, TOP ? 2 : 1), dim3(T), smem, st, TOP ? 2 : 1, a));
+    BFHE_LAUNCH_CHECK("k_ntt_fwd");
     return BFHE_OK;
 }
 
@@ -475,25 +460,8 @@ int run_inv(const NttArgs& a, int blocks, cudaStream_t st) {
                                        (int)smem));
         attr.fetch_or(1ull << dev);
     }
-    if (MODE == 2) {
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3(blocks, 2, 1);
-        cfg.blockDim = dim3(T, 1, 1);
-        cfg.dynamicSmemBytes = smem;
-        cfg.stream = st;
-        cudaLaunchAttribute at[1];
-        at[0].id = cudaLaunchAttributeClusterDimension;
-        at[0].val.clusterDim.x = 1;
-        at[0].val.clusterDim.y = 2;
-        at[0].val.clusterDim.z = 1;
-        cfg.attrs = at;
-        cfg.numAttrs = 1;
-        BFHE_CUDA(cudaLaunchKernelEx(&cfg, k_ntt_inv<PM, LOG_M, LOG_E, MODE, OUT>, a));
-        BFHE_LAUNCH_CHECK("k_ntt_inv (cluster)");
-    } else {
-        k_ntt_inv<PM, LOG_M, LOG_E, MODE, OUT><<<dim3(blocks, 1), T, smem, st>>>(a);
-        BFHE_LAUNCH_CHECK("k_ntt_inv");
-    }
+    BFHE_CUDA(launch_kernel(k_ntt_inv<PM, LOG_M, LOG_E, MODE, OUT>, dim3(blocks, (MODE == 2) ? 2 : 1), dim3(T), smem, st, (MODE == 2) ? 2 : 1, a));
+    BFHE_LAUNCH_CHECK("k_ntt_inv");
     return BFHE_OK;
 }
 
