@@ -163,6 +163,17 @@ __device__ __forceinline__ u64 pm_canon(u64 x, u64 q, int b, uint32_t d) {
     const u64 y = pm_lazy(x, q, b, d);
     return y >= q ? y - q : y;
 }
+// Sums of products of run-time factors x, y cut at bit hs = (b + 2) / 2 (x = x1 2^hs + x0): p00, pm, p11 the sums of
+// x0 y0, x0 y1 + x1 y0, x1 y1, below 2^61 and p11 2^(2 hs - b) below 2^60.  With H = floor(pm / 2^(b - hs)) +
+// p11 2^(2 hs - b) the sum is p00 + (pm mod 2^(b - hs)) 2^hs + H 2^b, folded by H 2^b = H d twice: signed, below 2^62.
+__device__ __forceinline__ u64 pm_fold3(u64 p00, u64 pm, u64 p11, int b, uint32_t d) {
+    const int hs = (b + 2) >> 1, s = b - 32;
+    const u64 H = (pm >> (b - hs)) + (p11 << (2 * hs - b));
+    const u64 g = (u64)(uint32_t)(H >> 32) * d;   // weight 2^32
+    u64 r = p00 + ((pm & (((u64)1 << (b - hs)) - 1)) << hs) + ((u64)((uint32_t)g & ((1u << s) - 1u)) << 32);
+    r = mad_wide_u((uint32_t)H, d, r);
+    return mad_wide_u((uint32_t)(g >> s), d, r);
+}
 // a b mod q, canonical, for two run-time factors below 2^(bits+1): the 128-bit product folded three times (eight wide
 // multiplies against Montgomery's ten and their carries)
 __device__ __forceinline__ u64 pm_mul_var(u64 a, u64 b, u64 q, int bits, uint32_t d) {
@@ -284,6 +295,10 @@ struct bfhe_ctx {
     PmSum pm_up, pm_toB, pm_toQ;
     PmDec pm_dec;
     const ulonglong2* d_xtw = nullptr;
+    // the same contexts' rounding division by P: twists N^-1 psi^-k P^-1 (data) and N^-1 psi^-k (special) [L + alpha][N],
+    // and the constants of the special digits [L][alpha]: -P^-1, then -p_0 P^-1 (words cut at b - 28).  Their tensor and
+    // key-switch inner product leave plain residues (no Montgomery factor).
+    const ulonglong2 *d_mtw = nullptr, *d_mpc = nullptr;
     // Shoup pair tables: p[i] = w_i, p[n + i] = ws_i
     const u64* d_tmod = nullptr;    // [nP] [t]_{prime}
     const u64* d_delta_q = nullptr; // [L]  [Delta]_{q_i}

@@ -533,12 +533,12 @@ extern "C" int bfhe_ctx_create(const bfhe_params* prm, int device, bfhe_ctx** ou
 
     // Products as pm_mul (common.cuh) when every transform stays below 2^63 in magnitude: one stage adds at most
     // 3 2^29 4d + 2.5 2^(bits + 2); the forward starts below 2^60 (the lift's sums, 2^(bits + 1) above 52 bits), the
-    // inverse's first pass sums up to 32 inputs.
+    // inverse's first pass sums up to 32 inputs (below 2^bits + 2^(63 - bits) d each).
     if (bits >= 45 && bits <= 55) {
         u64 d = 0;
         for (u64 q : rule.moduli) d = std::max(d, ((u64)1 << bits) - q);
         const u128 g = (u128)6442450944ull * d + ((u128)5 << (bits + 1));
-        c->pm = (u128)c->logN * g + ((u128)1 << (bits > 52 ? bits + 5 : 60)) < ((u128)1 << 63);
+        c->pm = (u128)c->logN * g + ((u128)1 << (bits > 52 ? bits + 5 : 60)) + ((u128)1 << 45) < ((u128)1 << 63);
     }
     // bit reversal
     c->brv.resize(N);
@@ -622,9 +622,11 @@ extern "C" int bfhe_ctx_create(const bfhe_params* prm, int device, bfhe_ctx** ou
         }
         // twist N^-1 psi^-m: plain, times R, and times t R (scale-and-round takes the multiply's inverse
         // transforms untwisted and folds the twist into its own product by t)
+        // (a context whose tensor leaves plain residues takes row 2 without R)
         const u64 ninv = invmod(N % q, q), tq = t % q;
+        const bool plain = pm_ctx && L <= BFHE_MAX_L_UNROLLED;
         for (uint32_t m = 0; m < N; ++m) {
-            const u64 v0 = mulmod(ninv, ipw[m], q), v1 = mulmod(v0, R, q), v2 = mulmod(v1, tq, q);
+            const u64 v0 = mulmod(ninv, ipw[m], q), v1 = mulmod(v0, R, q), v2 = mulmod(plain ? v0 : v1, tq, q);
             const u64 vs[3] = {v0, v1, v2};
             for (int f = 0; f < 3; ++f) {
                 const size_t o = (((size_t)p * 3 + f) * N + m) * 2;
@@ -649,7 +651,7 @@ extern "C" int bfhe_ctx_create(const bfhe_params* prm, int device, bfhe_ctx** ou
                      ePQ = build_ext(ar, Pp, Qp), eQt = build_ext(ar, Qp, Tp);
 
     // the same extensions for moduli 2^b - d
-    size_t o_xtw = 0;
+    size_t o_xtw = 0, o_mtw = 0, o_mpc = 0;
     const bool pm_ext = c->pm && L <= BFHE_MAX_L_UNROLLED;
     if (pm_ext) {
         const int b = (int)bits, hs = (b + 2) / 2;
@@ -700,17 +702,34 @@ extern "C" int bfhe_ctx_create(const bfhe_params* prm, int device, bfhe_ctx** ou
             c->pm_dec.c.push_back((uint32_t)ci);
             c->pm_dec.c2.push_back((uint32_t)mulmod(ci, ((u64)1 << hs) % t, t));
         }
-        // twist rows: t R N^-1 psi^-k of row 2 times the folded constant
+        // mod-down: twists times P^-1 over Q, plain over P, and the special digits' constants
+        std::vector<u64> mtw((size_t)(L + A) * N * 2), mpc((size_t)L * A * 2);
+        const u64 mask30 = ((u64)1 << (bits - 30)) - 1;
+        auto word = [&](size_t o) { return (twist[o] & mask30) | ((twist[o] >> 32) << (bits - 30)); };   // an entry's constant
+        for (uint32_t l = 0; l < L + A; ++l) {
+            const u64 q = c->primes[l];
+            const u64 f = l < L ? invmod(part(Pp, -1, q), q) : 1;
+            for (uint32_t m = 0; m < N; ++m) {
+                const size_t x = ((size_t)l * N + m) * 2;
+                pm_entry(mulmod(word(((size_t)l * 3 * N + m) * 2), f, q), q, b - 28, &mtw[x], &mtw[x + 1]);
+            }
+            if (l < L)
+                for (uint32_t a = 0; a < A; ++a) {
+                    const u64 g = a ? mulmod(f, Pp[0] % q, q) : f;
+                    pm_entry(q - g, q, b - 28, &mpc[(l * A + a) * 2], &mpc[(l * A + a) * 2 + 1]);
+                }
+        }
+        o_mtw = ar.add(mtw);
+        o_mpc = ar.add(mpc);
+        // twist rows: t N^-1 psi^-k of row 2 times the folded constant
         std::vector<u64> xtw((size_t)(L + K) * N * 2);
         for (uint32_t l = 0; l < L + K; ++l) {
             const uint32_t p = l < L ? l : l + A;
             const u64 q = c->primes[p];
             for (uint32_t m = 0; m < N; ++m) {
                 const size_t o = (((size_t)p * 3 + 2) * N + m) * 2;
-                const u64 mask = ((u64)1 << (bits - 30)) - 1;
-                const u64 w = (twist[o] & mask) | ((twist[o] >> 32) << (bits - 30));   // the entry's constant
                 const size_t x = ((size_t)l * N + m) * 2;
-                pm_entry(mulmod(w, fold[l], q), q, b - 28, &xtw[x], &xtw[x + 1]);
+                pm_entry(mulmod(word(o), fold[l], q), q, b - 28, &xtw[x], &xtw[x + 1]);
             }
         }
         o_xtw = ar.add(xtw);
@@ -776,7 +795,11 @@ extern "C" int bfhe_ctx_create(const bfhe_params* prm, int device, bfhe_ctx** ou
     c->ext_BQ = ext_ptrs(base, eBQ);
     c->ext_PQ = ext_ptrs(base, ePQ);
     c->ext_Qt = ext_ptrs(base, eQt);
-    if (pm_ext) c->d_xtw = reinterpret_cast<const ulonglong2*>(base + o_xtw);
+    if (pm_ext) {
+        c->d_xtw = reinterpret_cast<const ulonglong2*>(base + o_xtw);
+        c->d_mtw = reinterpret_cast<const ulonglong2*>(base + o_mtw);
+        c->d_mpc = reinterpret_cast<const ulonglong2*>(base + o_mpc);
+    }
     // the guarded fast extension of ext.cu measures faster from 8 data primes up (slower at 2); that of ext_pm.cu, for
     // moduli 2^b - d, at every size (64 pairs, lift + scale-and-round: N = 4096, L = 2: 61 -> 43 us, N = 8192, L = 4:
     // 242 -> 138), so it also replaces the mixed-radix path where the setting is off by default

@@ -9,6 +9,8 @@
 //
 // The exact base extensions (lift, scale-and-round, mod-down, decryption's
 // last step) are in ext.cu.
+#include <algorithm>
+
 #include "kernels.cuh"
 
 namespace {
@@ -135,6 +137,43 @@ __device__ __forceinline__ void tensor_word(u64 a0, u64 a1, u64 b0, u64 b1, u64 
     mac128(hi, lo, a1, b0);
     d1 = redc(hi, lo, q, qinv);
     d2 = redc(__umul64hi(a1, b1), a1 * b1, q, qinv);
+}
+
+// the same words with moduli 2^b - d: inputs below 2^(b+1), outputs plain residues (signed, within 2^(63-b) d of [0, 2^b)),
+// each sum folded instead of reduced by Montgomery's ten further multiplies (28 wide multiplies per word against 46: 64
+// pairs at N = 16384, L = 8 166 -> 149 us, 6.1 TB/s)
+__device__ __forceinline__ void tensor_word_pm(u64 a0, u64 a1, u64 b0, u64 b1, int b, uint32_t d, u64& d0, u64& d1, u64& d2) {
+    const int hs = (b + 2) >> 1;
+    const uint32_t mask = (1u << hs) - 1u;
+    const uint32_t a0l = (uint32_t)a0 & mask, a0h = (uint32_t)(a0 >> hs), a1l = (uint32_t)a1 & mask, a1h = (uint32_t)(a1 >> hs);
+    const uint32_t b0l = (uint32_t)b0 & mask, b0h = (uint32_t)(b0 >> hs), b1l = (uint32_t)b1 & mask, b1h = (uint32_t)(b1 >> hs);
+    d0 = pm_fold(pm_fold3((u64)a0l * b0l, mad_wide_u(a0h, b0l, (u64)a0l * b0h), (u64)a0h * b0h, b, d), b, d);
+    d2 = pm_fold(pm_fold3((u64)a1l * b1l, mad_wide_u(a1h, b1l, (u64)a1l * b1h), (u64)a1h * b1h, b, d), b, d);
+    u64 pm = (u64)a0l * b1h;
+    pm = mad_wide_u(a0h, b1l, pm);
+    pm = mad_wide_u(a1l, b0h, pm);
+    pm = mad_wide_u(a1h, b0l, pm);
+    d1 = pm_fold(pm_fold3(mad_wide_u(a1l, b0l, (u64)a0l * b1l), pm, mad_wide_u(a1h, b0h, (u64)a0h * b1h), b, d), b, d);
+}
+
+// tensor (SQ: squaring, b = a) in place as k_tensor; a block of 256 threads takes 512 words of one limb
+template <bool SQ>
+__global__ void __launch_bounds__(256) k_tensor_pm(u64* X, int LK, LimbMap map, PrimeTab tab, int logN, int b) {
+    pdl_next();
+    const int sh = logN - 9;
+    const uint32_t row = blockIdx.x >> sh, c = row / (uint32_t)LK, limb = row - c * LK;
+    const uint32_t d = (uint32_t)(((u64)1 << b) - tab.q[map((int)limb)]);
+    const size_t p2 = ((size_t)LK << logN) / 2;   // one plane in 16-byte units
+    ulonglong2* x = reinterpret_cast<ulonglong2*>(X + ((size_t)(c * 4 * LK + limb) << logN)) +
+                    (blockIdx.x & ((1u << sh) - 1u)) * 256 + threadIdx.x;
+    pdl_wait();
+    const ulonglong2 a0 = x[0], a1 = x[p2], b0 = SQ ? a0 : x[2 * p2], b1 = SQ ? a1 : x[3 * p2];
+    u64 e0, e1, e2, f0, f1, f2;
+    tensor_word_pm(a0.x, a1.x, b0.x, b1.x, b, d, e0, e1, e2);
+    tensor_word_pm(a0.y, a1.y, b0.y, b1.y, b, d, f0, f1, f2);
+    x[0] = make_ulonglong2(e0, f0);
+    x[p2] = make_ulonglong2(e1, f1);
+    x[2 * p2] = make_ulonglong2(e2, f2);
 }
 
 __global__ void k_tensor(u64* X, int n, int LK, LimbMap map, PrimeTab tab, int N) {
@@ -275,6 +314,83 @@ __global__ void __launch_bounds__(256, 2) k_inner(const u64* Dg, const u64* rlk,
             for (int b = 0; b < D; ++b)
 #pragma unroll
                 for (int j = 0; j < L; ++j) buf[b][j] = buf[b + 1][j];
+        }
+    }
+}
+
+// the same inner product for moduli 2^b - d: digits below 2^(b+1) and key words cut at bit hs, the three limb sums in
+// 64 bits, one fold per output, plain residues out (no Montgomery factor).  Up to 8 primes the middle sum comes from
+// (x0 + x1)(y0 + y1), three products per term with the key words' sums kept in registers; above, four.  The kernel with
+// Montgomery's reduction was bound by the multiplier pipe (97%): 28 instead of 42 multiplies per output at L = 8, where
+// it now waits on its digit loads (64 ciphertexts at N = 16384: 172 -> 158 us, 5.4 TB/s).
+template <int L>
+__global__ void __launch_bounds__(256, 2) k_inner_pm(const u64* __restrict__ Dg, const u64* __restrict__ rlk, u64* __restrict__ W,
+                                                     int n, int QP, int cpg, PrimeTab tab, int logN, int b) {
+    pdl_begin();
+    constexpr bool KARA = L <= 8;
+    constexpr int D = L <= 8 ? 2 : 0;   // ciphertexts of look-ahead
+    const int hs = (b + 2) >> 1;
+    const uint32_t mask = (1u << hs) - 1u;
+    const size_t plane = (size_t)QP << logN;
+    const int groups = (n + cpg - 1) / cpg;
+    const size_t total = plane * groups;
+    for (size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
+         idx += (size_t)gridDim.x * blockDim.x) {
+        const uint32_t row = (uint32_t)(idx >> logN), grp = row / (uint32_t)QP, k = row - grp * QP;
+        const size_t off = ((size_t)k << logN) + (idx & (((size_t)1 << logN) - 1));
+        const u64 q = tab.q[k];
+        const uint32_t d = (uint32_t)(((u64)1 << b) - q);
+        uint32_t yl[2][L], yh[2][L], ys[2][KARA ? L : 1];
+#pragma unroll
+        for (int j = 0; j < L; ++j)
+#pragma unroll
+            for (int m = 0; m < 2; ++m) {
+                const u64 y = __ldg(rlk + ((size_t)j * 2 + m) * plane + off);
+                yl[m][j] = (uint32_t)y & mask;
+                yh[m][j] = (uint32_t)(y >> hs);
+                if constexpr (KARA) ys[m][j] = yl[m][j] + yh[m][j];
+            }
+        const int c0 = grp * cpg, c_end = min(n, (int)(grp + 1) * cpg);
+        u64 buf[D + 1][L];
+#pragma unroll
+        for (int p = 0; p < D; ++p) {
+            if (c0 + p < c_end) {
+                const u64* s = Dg + (size_t)(c0 + p) * L * plane + off;
+#pragma unroll
+                for (int j = 0; j < L; ++j) buf[p][j] = s[(size_t)j * plane];
+            }
+        }
+        for (int c = c0; c < c_end; ++c) {
+            if (c + D < c_end) {
+                const u64* s = Dg + (size_t)(c + D) * L * plane + off;
+#pragma unroll
+                for (int j = 0; j < L; ++j) buf[D][j] = s[(size_t)j * plane];
+            }
+            u64 p00[2] = {0, 0}, pm[2] = {0, 0}, p11[2] = {0, 0};
+#pragma unroll
+            for (int j = 0; j < L; ++j) {
+                const uint32_t xl = (uint32_t)buf[0][j] & mask, xh = (uint32_t)(buf[0][j] >> hs);
+#pragma unroll
+                for (int m = 0; m < 2; ++m) {
+                    p00[m] += (u64)xl * yl[m][j];
+                    p11[m] += (u64)xh * yh[m][j];
+                    if constexpr (KARA) {
+                        pm[m] += (u64)(xl + xh) * ys[m][j];
+                    } else {
+                        pm[m] += (u64)xl * yh[m][j];
+                        pm[m] += (u64)xh * yl[m][j];
+                    }
+                }
+            }
+#pragma unroll
+            for (int m = 0; m < 2; ++m) {
+                if constexpr (KARA) pm[m] -= p00[m] + p11[m];
+                W[((size_t)c * 2 + m) * plane + off] = pm_fold(pm_fold3(p00[m], pm[m], p11[m], b, d), b, d);
+            }
+#pragma unroll
+            for (int p = 0; p < D; ++p)
+#pragma unroll
+                for (int j = 0; j < L; ++j) buf[p][j] = buf[p + 1][j];
         }
     }
 }
@@ -673,6 +789,13 @@ int launch_tensor(const bfhe_ctx* ctx, u64* X, int n, int square, cudaStream_t s
     ProfScope ps(ctx, BFHE_K_TENSOR, st, 4.0 * n * (ctx->L + ctx->K) * ctx->N,
                  (square ? 40.0 : 56.0) * n * (ctx->L + ctx->K) * ctx->N);
     const int LK = (int)(ctx->L + ctx->K);
+    if (ctx->pm_ext) {
+        const dim3 grid((unsigned)((size_t)n * LK << (ctx->logN - 9)));
+        BFHE_CUDA(launch_kernel(square ? k_tensor_pm<true> : k_tensor_pm<false>, grid, dim3(256), 0, st, 1, X, LK, ctx->mapQB(),
+                                ctx->tab, (int)ctx->logN, (int)ctx->prime_bits));
+        BFHE_LAUNCH_CHECK("k_tensor_pm");
+        return BFHE_OK;
+    }
     if (square)
         LAUNCH(k_tensor_sq, (size_t)n * LK * ctx->N / 2, X, n, LK, ctx->mapQB(), ctx->tab, (int)ctx->N);
     else
@@ -683,9 +806,16 @@ int launch_tensor(const bfhe_ctx* ctx, u64* X, int n, int square, cudaStream_t s
 template <int L>
 int run_inner(const bfhe_ctx* ctx, const u64* Dg, u64* W, int n, cudaStream_t st) {
     const int QP = (int)(ctx->L + ctx->alpha);
-    const int cpg = n < 4 ? 1 : (n + 3) / 4;   // four groups: enough threads, key read four times
-    const size_t work = (size_t)QP * ctx->N * ((n + cpg - 1) / cpg);
-    if (ctx->prime_bits <= 50)   // digits below 64q < 2^56 (lazy transforms), key words below 2^50
+    // The key is read once per group of ciphertexts: as few groups as give four waves of two blocks per SM.  (A fixed four
+    // read the 151 MB key of N = 32768, L = 16 four times, half of the kernel's traffic: 236 -> 175 us for 8 ciphertexts;
+    // N = 4096, L = 2 left half of the SMs idle: 13 -> 12 us for 64.)
+    const size_t plane = (size_t)QP * ctx->N, want = (size_t)4 * 152 * 2 * TPB;
+    const int groups = (int)std::min<size_t>((size_t)n, std::max<size_t>(1, (want + plane - 1) / plane));
+    const int cpg = (n + groups - 1) / groups;
+    const size_t work = plane * ((n + cpg - 1) / cpg);
+    if (ctx->pm_ext)
+        LAUNCH(k_inner_pm<L>, work, Dg, ctx->d_rlk_ntt, W, n, QP, cpg, ctx->tab, (int)ctx->logN, (int)ctx->prime_bits);
+    else if (ctx->prime_bits <= 50)   // digits below 64q < 2^56 (lazy transforms), key words below 2^50
         LAUNCH((k_inner<L, true>), work, Dg, ctx->d_rlk_ntt, W, n, QP, cpg, ctx->tab, (int)ctx->N);
     else
         LAUNCH((k_inner<L, false>), work, Dg, ctx->d_rlk_ntt, W, n, QP, cpg, ctx->tab, (int)ctx->N);

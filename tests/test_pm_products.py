@@ -224,3 +224,30 @@ def test_product_of_two_run_time_factors(bits):
             assert g < 1 << 64
             r = ((m & ((1 << s) - 1)) << 32 | lo & M) + ((g & ((1 << s) - 1)) << 32) + h0 * d + u32(g >> s) * d
             assert r < 1 << 63 and (r - a * b) % q == 0
+
+
+@pytest.mark.parametrize("bits", [45, 50, 51, 55])
+@pytest.mark.parametrize("terms", [1, 2, 8, 16])
+def test_limb_sums_fold_to_the_sum_of_products(bits, terms):
+    """pm_fold3 on the three limb sums of x y (x below 2^(bits+1), y below 2^bits; with (x0 + x1)(y0 + y1) as well):
+    no sum wraps, the fold is congruent and below 2^62."""
+    rng = random.Random(bits + terms)
+    q = Params(N=32768, L=16, alpha=2, prime_bits=bits).b[-1]
+    d, hs, s, M = (1 << bits) - q, (bits + 2) // 2, bits - 32, (1 << 32) - 1
+    mask = (1 << hs) - 1
+    for case in range(40):
+        xs = [(2 << bits) - 1 if case == 0 else rng.randrange(2 << bits) for _ in range(terms)]
+        ys = [(2 << bits) - 1 if case == 0 and terms <= 2 else q - 1 if case == 0 else rng.randrange(q) for _ in range(terms)]
+        p00 = pm = p11 = pk = 0
+        for x, y in zip(xs, ys):
+            x0, x1, y0, y1 = u32(x & mask), u32(x >> hs), u32(y & mask), u32(y >> hs)
+            p00, pm, p11 = p00 + x0 * y0, pm + x0 * y1 + x1 * y0, p11 + x1 * y1
+            pk += u32(x0 + x1) * u32(y0 + y1)
+        assert pk - p00 - p11 == pm
+        if terms <= 8:
+            assert pk < 1 << 64
+        assert max(p00, pm, p11) <= 1 << 61 and p11 << (2 * hs - bits) <= 1 << 60
+        H = (pm >> (bits - hs)) + (p11 << (2 * hs - bits))
+        g = u32(H >> 32) * d
+        r = p00 + ((pm & ((1 << (bits - hs)) - 1)) << hs) + ((g & ((1 << s) - 1)) << 32) + (H & M) * d + u32(g >> s) * d
+        assert r < 1 << 62 and (r - sum(x * y for x, y in zip(xs, ys))) % q == 0
