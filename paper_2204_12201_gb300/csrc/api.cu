@@ -10,6 +10,8 @@ namespace {
 // Philox purposes (key word 1)
 enum : u64 { P_SK = 1, P_PK_A = 2, P_PK_E = 3, P_RLK_A = 4, P_RLK_E = 5, P_ENC_U = 6, P_ENC_E1 = 7, P_ENC_E2 = 8 };
 
+inline bool aligned16(const void* p) { return ((uintptr_t)p & 15) == 0; }
+
 inline cudaStream_t S(void* s) { return (cudaStream_t)s; }
 
 // device-memory budget for one call's scratch (batches beyond it are tiled)
@@ -36,8 +38,9 @@ size_t mul_words_per_ct(const bfhe_ctx* c) { return mul_scratch_bytes(c, 1) / si
 size_t g_mul_tile[16] = {};
 
 // out[i] = a[i] * b[i] (relinearised), n ciphertexts, scratch of `scratch_words` words
+// epi (pm_ext contexts): the products go through a gate equation instead of to out
 int mul_relin_impl(bfhe_ctx* c, const u64* A, const u64* B, u64* out, size_t n, u64* scratch,
-                   size_t scratch_words, cudaStream_t st) {
+                   size_t scratch_words, cudaStream_t st, const MulEpilogue* epi = nullptr) {
     const size_t N = c->N, L = c->L, K = c->K, LK = L + K, QP = L + c->alpha;
     const size_t per = mul_words_per_ct(c);
     size_t tile = scratch_words / per;
@@ -93,7 +96,13 @@ int mul_relin_impl(bfhe_ctx* c, const u64* A, const u64* B, u64* out, size_t n, 
         RC(launch_ntt_fwd(c, iod, m * (int)L, (int)QP, c->mapQP(), st, 1));   // so does the inner product
         RC(launch_inner(c, Dg, W, m, st));
         RC(launch_ntt_inv(c, ntt_io(W, W, QP, N), 2 * m, (int)QP, c->mapQP(), 1, st, 2));   // so does mod-down
-        RC(launch_moddown(c, W, C3, o, m, st));
+        if (epi) {
+            MulEpilogue e = *epi;
+            e.c0 = (uint32_t)c0;
+            RC(launch_moddown(c, W, C3, o, m, st, &e));
+        } else {
+            RC(launch_moddown(c, W, C3, o, m, st));
+        }
     }
     return BFHE_OK;
 }
@@ -577,16 +586,28 @@ extern "C" int bfhe_bit_gate(bfhe_ctx* c, int gate, const uint64_t* x, const uin
         u64 *fixed, *mul;
         size_t mw;
         const bool mux = gate == BFHE_MUX;
-        RC(scratch_for(c, (mux ? 2 : 1) * n * ctw, n, &fixed, &mul, &mw));
+        // the multiply's last kernel applies the gate equation when it reads the operands in 16-byte words
+        const bool fused = c->pm_ext && n < ((size_t)1 << 31) && aligned16(x) && aligned16(y) && (!z || aligned16(z)) && aligned16(out);
+        RC(scratch_for(c, ((mux ? 1 : 0) + (fused ? 0 : 1)) * n * ctw, n, &fixed, &mul, &mw));
         u64* P = fixed;
         const u64* rhs = y;
         if (mux) {
-            u64* D = fixed + n * ctw;
+            u64* D = fixed + (fused ? 0 : n * ctw);
             RC(launch_lincomb(c, D, y, z, nullptr, nullptr, LinCoef{0, 1, -1, 0, 0}, 0, n, st));
             rhs = D;
         }
-        RC(mul_relin_impl(c, x, rhs, P, n, mul, mw, st));
-        RC(launch_lincomb(c, out, x, y, z, P, kGate[gate], 1, n, st));
+        if (fused) {
+            MulEpilogue epi;
+            epi.kind = 1;
+            epi.cf = kGate[gate];
+            epi.x = x;
+            epi.y = y;
+            epi.z = z;
+            RC(mul_relin_impl(c, x, rhs, out, n, mul, mw, st, &epi));
+        } else {
+            RC(mul_relin_impl(c, x, rhs, P, n, mul, mw, st));
+            RC(launch_lincomb(c, out, x, y, z, P, kGate[gate], 1, n, st));
+        }
         c->counts[2] += n;
     }
     c->counts[0] += n * kGateAddSub[gate][0];
@@ -605,12 +626,25 @@ extern "C" int bfhe_gate_level(bfhe_ctx* c, uint64_t* wires, size_t n_wires, siz
         CHECK_KEYS(c);
         u64 *fixed, *mul;
         size_t mw;
-        RC(scratch_for(c, 3 * n_mul * ctw, n_mul * n, &fixed, &mul, &mw));
+        const bool fused = c->pm_ext && n_mul * n < ((size_t)1 << 31) && aligned16(wires);
+        RC(scratch_for(c, (fused ? 2 : 3) * n_mul * ctw, n_mul * n, &fixed, &mul, &mw));
         u64* AB = fixed;
         u64* P = fixed + 2 * n_mul * ctw;
         RC(launch_gather(c, AB, wires, n, table, (int)n_mul, st));
-        RC(mul_relin_impl(c, AB, AB + n_mul * ctw, P, n_mul * n, mul, mw, st));
-        RC(launch_gate_epilogue(c, wires, n, table, (int)n_gates, P, (int)n_mul, st));
+        if (fused) {
+            // products go through their entries' equations to the wires; the linear entries read none of those
+            MulEpilogue epi;
+            epi.kind = 2;
+            epi.wires = wires;
+            epi.table = table;
+            epi.n = (uint32_t)n;
+            RC(mul_relin_impl(c, AB, AB + n_mul * ctw, wires, n_mul * n, mul, mw, st, &epi));
+            if (n_gates > n_mul)
+                RC(launch_gate_epilogue(c, wires, n, table + 5 * n_mul, (int)(n_gates - n_mul), nullptr, 0, st));
+        } else {
+            RC(mul_relin_impl(c, AB, AB + n_mul * ctw, P, n_mul * n, mul, mw, st));
+            RC(launch_gate_epilogue(c, wires, n, table, (int)n_gates, P, (int)n_mul, st));
+        }
         c->counts[2] += n_mul * n;
     } else {
         RC(launch_gate_epilogue(c, wires, n, table, (int)n_gates, nullptr, 0, st));

@@ -10,6 +10,7 @@
 // count with a mixed-radix fallback near the rounding boundary).  Both give
 // the same integers.
 #include "ext_device.cuh"
+#include "rows.cuh"
 
 namespace {
 
@@ -370,10 +371,11 @@ __device__ __forceinline__ u64 fold28(u64 P, u64 Q, int b, uint32_t d) {
     return mad_wide_s((int)(Q >> 32), (int)(d << 4), add64(P, ((u64)(ql >> (32 - k)) << 32) | (ql << k)));
 }
 
-template <int NA>
-__global__ void __launch_bounds__(256) k_moddown_pm(const u64* __restrict__ W, const u64* __restrict__ C3, u64* __restrict__ out,
+template <int NA, bool EPI>
+__global__ void __launch_bounds__(256) k_moddown_pm(const u64* __restrict__ W, const u64* __restrict__ C3, u64* out,
                                                     int L, ExtDesc ePQ, const ulonglong2* __restrict__ mtw,
-                                                    const ulonglong2* __restrict__ mpc, const u64* __restrict__ qtab, int logN, int b) {
+                                                    const ulonglong2* __restrict__ mpc, const u64* __restrict__ qtab, int logN, int b,
+                                                    MulEpilogue epi, const u64* __restrict__ delta) {
     pdl_next();
     // a block takes 512 coefficients of one polynomial
     const int sh = logN - 9;
@@ -398,6 +400,28 @@ __global__ void __launch_bounds__(256) k_moddown_pm(const u64* __restrict__ W, c
     const u64 neg0 = garner<NA>(x0, ePQ, v0) ? 1 : 0, neg1 = garner<NA>(x1, ePQ, v1) ? 1 : 0;
     const u64* cin = C3 + ((size_t)(c * 3 + comp) * L << logN) + k;
     u64* o = out + ((size_t)cp * L << logN) + k;
+    // EPI: the operands' words sit where the product's would, shifted to their wires for a table entry
+    LinCoef cf{};
+    const u64 *ex = nullptr, *ey = nullptr, *ez = nullptr;
+    if constexpr (EPI) {
+        const uint32_t cg = epi.c0 + c;
+        if (epi.kind == 1) {
+            cf = epi.cf;
+            const size_t at = ((size_t)(2 * cg + comp) * L << logN) + k;
+            ex = epi.x + at;
+            ey = epi.y + at;
+            ez = epi.z + at;
+        } else {
+            const uint32_t g = cg / epi.n, ci = cg - g * epi.n;
+            const int32_t* t = epi.table + 5 * g;
+            gate_coefs(t[0], cf.cc, cf.cx, cf.cy, cf.cz, cf.cp);
+            const size_t ctw = (size_t)epi.n * 2 * L << logN, at = ((size_t)(2 * ci + comp) * L << logN) + k;
+            ex = epi.wires + (size_t)t[1] * ctw + at;
+            ey = epi.wires + (size_t)t[2] * ctw + at;
+            ez = epi.wires + (size_t)t[3] * ctw + at;
+            o = epi.wires + (size_t)t[4] * ctw + at;
+        }
+    }
 #pragma unroll 4
     for (int i = 0; i < L; ++i) {
         const u64 q = qtab[i];
@@ -414,8 +438,23 @@ __global__ void __launch_bounds__(256) k_moddown_pm(const u64* __restrict__ W, c
             mul28(v0[a], e, P0, Q0);
             mul28(v1[a], e, P1, Q1);
         }
-        *reinterpret_cast<ulonglong2*>(o + ((size_t)i << logN)) =
-            make_ulonglong2(pm_canon(fold28(P0, Q0, b, d), q, b, d), pm_canon(fold28(P1, Q1, b, d), q, b, d));
+        u64 r0 = pm_canon(fold28(P0, Q0, b, d), q, b, d), r1 = pm_canon(fold28(P1, Q1, b, d), q, b, d);
+        const size_t l = (size_t)i << logN;
+        if constexpr (EPI) {
+            Words<2> acc{};
+            if (cf.cc && comp == 0 && k == 0) acc.v[0] = apply(0, delta[i], cf.cc, q);   // the constant 1
+            auto term = [&](const u64* s, int m) {
+                const Words<2> t = load_words<2>(s);
+                acc.v[0] = apply(acc.v[0], t.v[0], m, q);
+                acc.v[1] = apply(acc.v[1], t.v[1], m, q);
+            };
+            if (cf.cx) term(ex + l, cf.cx);
+            if (cf.cy) term(ey + l, cf.cy);
+            if (cf.cz) term(ez + l, cf.cz);
+            r0 = apply(acc.v[0], r0, cf.cp, q);
+            r1 = apply(acc.v[1], r1, cf.cp, q);
+        }
+        *reinterpret_cast<ulonglong2*>(o + l) = make_ulonglong2(r0, r1);
     }
 }
 
@@ -608,7 +647,9 @@ int launch_scale(const bfhe_ctx* ctx, const u64* X, u64* C3, int n, cudaStream_t
     return BFHE_OK;
 }
 
-int launch_moddown(const bfhe_ctx* ctx, const u64* W, const u64* C3, u64* out, int n, cudaStream_t st) {
+int launch_moddown(const bfhe_ctx* ctx, const u64* W, const u64* C3, u64* out, int n, cudaStream_t st,
+                   const MulEpilogue* epi) {
+    if (epi && !ctx->pm_ext) return set_error(BFHE_EINVAL, "no fused gate equation for these moduli");
     const double A_ = ctx->alpha;
     // work: the rounding division by P, plus the twist the inverse transform left to this kernel
     // per coefficient of each of 2 polys: L + alpha words of W and L of C3 read, L written
@@ -617,9 +658,11 @@ int launch_moddown(const bfhe_ctx* ctx, const u64* W, const u64* C3, u64* out, i
     const size_t work = (size_t)n * ctx->N;   // two coefficients per thread
     if (ctx->pm_ext) {
         const dim3 grid((unsigned)((size_t)n * 2 << (ctx->logN - 9)));
-        BFHE_CUDA(launch_kernel(ctx->alpha == 1 ? k_moddown_pm<1> : k_moddown_pm<2>, grid, dim3(256), 0, st, 1, W, C3, out,
-                                (int)ctx->L, ctx->ext_PQ, ctx->d_mtw, ctx->d_mpc, ctx->tab.q, (int)ctx->logN,
-                                (int)ctx->prime_bits));
+        auto* kern = epi ? (ctx->alpha == 1 ? k_moddown_pm<1, true> : k_moddown_pm<2, true>)
+                         : (ctx->alpha == 1 ? k_moddown_pm<1, false> : k_moddown_pm<2, false>);
+        BFHE_CUDA(launch_kernel(kern, grid, dim3(256), 0, st, 1, W, C3, out, (int)ctx->L, ctx->ext_PQ, ctx->d_mtw, ctx->d_mpc,
+                                ctx->tab.q, (int)ctx->logN, (int)ctx->prime_bits, epi ? *epi : MulEpilogue{},
+                                ctx->d_delta_q));
         BFHE_LAUNCH_CHECK("k_moddown_pm");
         return BFHE_OK;
     }

@@ -18,6 +18,22 @@ struct PwStrides {
 int launch_pointwise(const bfhe_ctx* ctx, const u64* A, const u64* B, u64* out, int n, int polys, int n_limbs,
                      LimbMap map, PwStrides s, cudaStream_t st);
 
+// linear combination: out = cc*Delta*[c0, coeff 0] + cx x + cy y + cz z + cp p (coefficients in -2..2)
+struct LinCoef {
+    int cc, cx, cy, cz, cp;
+};
+// What a multiply's last kernel does with the product words it holds, instead of storing them for another kernel: the
+// gate equation over x, y, z (kind 1, buffers laid out as the output) or a level's table entries over the wires (kind 2).
+struct MulEpilogue {
+    int kind = 0;
+    LinCoef cf{};
+    const u64 *x = nullptr, *y = nullptr, *z = nullptr;
+    u64* wires = nullptr;
+    const int32_t* table = nullptr;
+    uint32_t n = 1;    // ciphertexts per wire
+    uint32_t c0 = 0;   // this launch's first product in the batch
+};
+
 // exact multiply pipeline pieces
 // slots = 4 (a0 a1 b0 b1) or 2 (squaring: a0 a1 only)
 int launch_modup(const bfhe_ctx* ctx, const u64* A, const u64* B, u64* X, int n, int slots, cudaStream_t st);
@@ -29,7 +45,9 @@ int launch_tensor(const bfhe_ctx* ctx, u64* X, int n, int square, cudaStream_t s
 // tmp: [n][3][K][N] words for the two-pass form (10 or more data primes), or null for one pass
 int launch_scale(const bfhe_ctx* ctx, const u64* X, u64* C3, int n, cudaStream_t st, u64* tmp = nullptr);
 int launch_inner(const bfhe_ctx* ctx, const u64* Dg, u64* W, int n, cudaStream_t st);
-int launch_moddown(const bfhe_ctx* ctx, const u64* W, const u64* C3, u64* out, int n, cudaStream_t st);
+// epi: pm contexts of at most 16 primes only
+int launch_moddown(const bfhe_ctx* ctx, const u64* W, const u64* C3, u64* out, int n, cudaStream_t st,
+                   const MulEpilogue* epi = nullptr);
 
 // decrypt: V = [c1 s]_Q (coefficient form), ct -> M = [round(t (c0 + c1 s) / Q)]_t
 int launch_dec_finish(const bfhe_ctx* ctx, const u64* V, const u64* ct, u64* M, int n, cudaStream_t st);
@@ -42,10 +60,6 @@ int launch_enc_finish(const bfhe_ctx* ctx, u64* ct, const u64* M, const i64* e1,
 int launch_neg_add_small(const bfhe_ctx* ctx, const u64* as, const i64* e, u64* out, int n_polys, int n_limbs,
                          LimbMap map, const u64* s2, int gadget, cudaStream_t st);
 
-// linear combination: out = cc*Delta*[c0, coeff 0] + cx x + cy y + cz z + cp p (coefficients in -2..2)
-struct LinCoef {
-    int cc, cx, cy, cz, cp;
-};
 int launch_lincomb(const bfhe_ctx* ctx, u64* out, const u64* x, const u64* y, const u64* z, const u64* p,
                    LinCoef cf, u64 cval, size_t n, cudaStream_t st);
 int launch_mul_scalar(const bfhe_ctx* ctx, const u64* a, u64 c, u64* out, size_t n, cudaStream_t st);

@@ -39,3 +39,26 @@ def test_linear_calls_on_buffers_aligned_to_one_word():
     ref = (a.cpu() + b.cpu()) % q.cpu()
     assert torch.equal(want[0].cpu(), ref)
     ctx.close()
+
+
+def test_gates_on_buffers_aligned_to_one_word():
+    """Every gate with the equation fused into the multiply (16-byte aligned buffers) and as a kernel of its own."""
+    need_gpu()
+    import __graft_entry__
+    __graft_entry__.build()
+    from paper_2204_12201_gb300 import bfhe
+    for alpha, bits in ((1, 50), (2, 55), (1, 40)):
+        ctx = bfhe.Context(N=1024, L=2, alpha=alpha, prime_bits=bits)
+        ctx.keygen(3)
+        n = 3
+        x, y, z = (ctx.encrypt(torch.randint(0, 2, (n, ctx.N), device="cuda"), s) for s in (1, 2, 3))
+        px, py, pz = (ctx.decrypt(t) for t in (x, y, z))
+        flat = torch.empty(x.numel() + 1, dtype=torch.int64, device="cuda")[1:].view(x.shape)
+        want = {bfhe.AND: px & py, bfhe.OR: px | py, bfhe.XOR: px ^ py, bfhe.NAND: 1 - (px & py), bfhe.NOR: 1 - (px | py),
+                bfhe.XNOR: 1 - (px ^ py), bfhe.MUX: torch.where(px == 1, py, pz)}
+        for gate, w in want.items():
+            got = ctx.bit_gate(gate, x, y, z)
+            assert torch.equal(got, ctx.bit_gate(gate, x, y, z, out=flat))
+            if bits >= 50:   # noise budget for one product
+                assert torch.equal(ctx.decrypt(got), w)
+        ctx.close()
