@@ -192,9 +192,19 @@ __device__ __forceinline__ u64 pm_mul_var(u64 a, u64 b, u64 q, int bits, uint32_
     r = mad_wide_u((uint32_t)(g >> s), d, r);  // below 2^60
     return pm_canon(r, q, bits, d);
 }
+// host: x mod q for q = 2^b - d with d below 2^27 and x below 2^(2b) (folds; a 128-bit division takes several times longer
+// and a context's tables need one per entry)
+inline u64 pm_reduce(u128 x, u64 q) {
+    const int b = 64 - __builtin_clzll(q);
+    const u64 d = ((u64)1 << b) - q, mask = ((u64)1 << b) - 1;
+    while (x >> b) x = (x >> b) * d + ((u64)x & mask);
+    u64 r = (u64)x;
+    while (r >= q) r -= q;
+    return r;
+}
 // host: the table entry of w, cut at bit k (b - 30 for pm_mul)
 inline void pm_entry(u64 w, u64 q, int k, u64* x, u64* y) {
-    const u64 m = ((u64)1 << k) - 1, v = (u64)(((u128)w << 32) % q);
+    const u64 m = ((u64)1 << k) - 1, v = pm_reduce((u128)w << 32, q);
     *x = (w & m) | ((w >> k) << 32);
     *y = (v & m) | ((v >> k) << 32);
 }

@@ -579,12 +579,13 @@ extern "C" int bfhe_ctx_create(const bfhe_params* prm, int device, bfhe_ctx** ou
                 t[o + 1] = shoup_of(w, q);
             }
         };
+        auto mm = [&](u64 a, u64 b) { return pm ? pm_reduce((u128)a * b, q) : mulmod(a, b, q); };
         // powers psi^k and psi^-k, k < 2N
         std::vector<u64> pw(2 * N), ipw(2 * N);
         pw[0] = ipw[0] = 1;
         for (uint32_t k = 1; k < 2 * N; ++k) {
-            pw[k] = mulmod(pw[k - 1], psi, q);
-            ipw[k] = mulmod(ipw[k - 1], ipsi, q);
+            pw[k] = mm(pw[k - 1], psi);
+            ipw[k] = mm(ipw[k - 1], ipsi);
         }
         // forward: psi^brv(k)
         for (uint32_t k = 0; k < N; ++k) {
@@ -626,7 +627,7 @@ extern "C" int bfhe_ctx_create(const bfhe_params* prm, int device, bfhe_ctx** ou
         const u64 ninv = invmod(N % q, q), tq = t % q;
         const bool plain = pm_ctx && L <= BFHE_MAX_L_UNROLLED;
         for (uint32_t m = 0; m < N; ++m) {
-            const u64 v0 = mulmod(ninv, ipw[m], q), v1 = mulmod(v0, R, q), v2 = mulmod(plain ? v0 : v1, tq, q);
+            const u64 v0 = mm(ninv, ipw[m]), v1 = mm(v0, R), v2 = mm(plain ? v0 : v1, tq);
             const u64 vs[3] = {v0, v1, v2};
             for (int f = 0; f < 3; ++f) {
                 const size_t o = (((size_t)p * 3 + f) * N + m) * 2;
@@ -711,7 +712,7 @@ extern "C" int bfhe_ctx_create(const bfhe_params* prm, int device, bfhe_ctx** ou
             const u64 f = l < L ? invmod(part(Pp, -1, q), q) : 1;
             for (uint32_t m = 0; m < N; ++m) {
                 const size_t x = ((size_t)l * N + m) * 2;
-                pm_entry(mulmod(word(((size_t)l * 3 * N + m) * 2), f, q), q, b - 28, &mtw[x], &mtw[x + 1]);
+                pm_entry(pm_reduce((u128)word(((size_t)l * 3 * N + m) * 2) * f, q), q, b - 28, &mtw[x], &mtw[x + 1]);
             }
             if (l < L)
                 for (uint32_t a = 0; a < A; ++a) {
@@ -729,7 +730,7 @@ extern "C" int bfhe_ctx_create(const bfhe_params* prm, int device, bfhe_ctx** ou
             for (uint32_t m = 0; m < N; ++m) {
                 const size_t o = (((size_t)p * 3 + 2) * N + m) * 2;
                 const size_t x = ((size_t)l * N + m) * 2;
-                pm_entry(mulmod(word(o), fold[l], q), q, b - 28, &xtw[x], &xtw[x + 1]);
+                pm_entry(pm_reduce((u128)word(o) * fold[l], q), q, b - 28, &xtw[x], &xtw[x + 1]);
             }
         }
         o_xtw = ar.add(xtw);
