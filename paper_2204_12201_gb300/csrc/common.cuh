@@ -1,10 +1,11 @@
 // common.cuh -- shared definitions of the bfhe CUDA library (sm_103a).
 //
-// Exact 64-bit modular arithmetic for RNS BFV on the integer pipe: Shoup
-// products for multiplications by precomputed constants (twiddles, CRT
-// constants), Montgomery reduction (REDC) for products of two runtime values
-// and for lazily accumulated sums of them.  Every modulus is an odd prime
-// below 2^60; the NTT keeps values lazily in [0, 4q).
+// Exact 64-bit modular arithmetic for RNS BFV on the integer pipe: for moduli
+// 2^b - d of 45 to 55 bits, products and sums of products folded by 2^b = d;
+// otherwise Shoup products for multiplications by precomputed constants
+// (twiddles, CRT constants) and Montgomery reduction (REDC) for products of
+// two runtime values and for lazily accumulated sums of them.  Every modulus
+// is an odd prime below 2^60.
 #pragma once
 
 #include <cuda_runtime.h>

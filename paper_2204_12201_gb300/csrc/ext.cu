@@ -8,7 +8,8 @@
 // (k_dec_finish).  Extensions run Garner's mixed-radix conversion, or, when
 // the context enables it, the guarded fast conversion (a fixed-point overflow
 // count with a mixed-radix fallback near the rounding boundary).  Both give
-// the same integers.
+// the same integers.  Contexts with moduli 2^b - d of 45 to 55 bits and at most
+// 16 data primes take ext_pm.cu instead, and k_moddown_pm here.
 #include "ext_device.cuh"
 #include "rows.cuh"
 
