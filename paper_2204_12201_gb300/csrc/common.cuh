@@ -394,7 +394,9 @@ int cuda_check(cudaError_t e, const char* where);
 // Every kernel of the library starts with pdl_begin and is launched with launch_kernel: the launch of a kernel, its
 // blocks' arrival and its reads of constant tables overlap the tail of the one before it on the stream (programmatic
 // dependent launch), and nothing that an earlier kernel writes, or still reads, is touched before pdl_wait returns, which
-// is when that kernel has completed.  Measured on GB300, calls one after another: a multiply of one pair at N = 16384,
+// is when that kernel has completed.  A kernel's buffers therefore change while it is resident: only the tables made with
+// the context are read through __restrict__ or __ldg, whose loads the wait need not order; ciphertexts, scratch and keys
+// (which key generation's kernels write) are plain pointers.  Measured on GB300, calls one after another: a multiply of one pair at N = 16384,
 // L = 8 102 -> 81 us, of 64 pairs at N = 4096, L = 2 159 -> 145 us, of 64 at N = 16384 2510 -> 2491 us; one XOR gate at
 // N = 4096 53 -> 37 us.  Inside a CUDA graph the plain dependency is the cheaper one (16-bit comparator at N = 4096
 // replayed: 263 us, with programmatic edges 286), so a launch on a capturing stream leaves the attribute out.

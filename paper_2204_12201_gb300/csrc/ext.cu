@@ -373,7 +373,7 @@ __device__ __forceinline__ u64 fold28(u64 P, u64 Q, int b, uint32_t d) {
 }
 
 template <int NA, bool EPI>
-__global__ void __launch_bounds__(256) k_moddown_pm(const u64* __restrict__ W, const u64* __restrict__ C3, u64* out,
+__global__ void __launch_bounds__(256) k_moddown_pm(const u64* W, const u64* C3, u64* out,
                                                     int L, ExtDesc ePQ, const ulonglong2* __restrict__ mtw,
                                                     const ulonglong2* __restrict__ mpc, const u64* __restrict__ qtab, int logN, int b,
                                                     MulEpilogue epi, const u64* __restrict__ delta) {

@@ -150,7 +150,7 @@ __device__ __noinline__ void scale_exact(const u64* d, u64* o, int k, int N, int
 // folded below 2^(b+1) above
 template <int NS>
 __global__ void __launch_bounds__(256, NS <= 8 ? 4 : 2)
-    k_modup_pm(const u64* __restrict__ A, const u64* __restrict__ B, u64* __restrict__ X, int n, int slots, int logN, int b,
+    k_modup_pm(const u64* A, const u64* B, u64* X, int n, int slots, int logN, int b,
                ExtDesc ext, uint32_t* flags, const __grid_constant__ PrepTab<NS> p,
                const __grid_constant__ SumTab<NS, NS + 1> t) {
     pdl_begin();
@@ -251,7 +251,7 @@ __device__ __forceinline__ u64 scale_out(const Digits<NS + 1>& z, int v, const S
 // loop unrolled, so that the constants are operands and the digits stay in registers
 template <int NS>
 __global__ void __launch_bounds__(256, 2)
-    k_scale_pm(const u64* __restrict__ X, u64* __restrict__ C3, int n, int logN, int b, const ulonglong2* __restrict__ xtw,
+    k_scale_pm(const u64* X, u64* C3, int n, int logN, int b, const ulonglong2* __restrict__ xtw,
                const __grid_constant__ SumTab<NS, NS + 1> tq, const __grid_constant__ SumTab<NS + 1, NS> tb,
                const __grid_constant__ ExactScale ex) {
     pdl_begin();
@@ -295,7 +295,7 @@ constexpr u64 Z_EXACT = (u64)1 << 62;
 
 template <int NS>
 __global__ void __launch_bounds__(256, 2)
-    k_scale_pm_a(const u64* __restrict__ X, u64* __restrict__ Z, int n, int logN, int b, const ulonglong2* __restrict__ xtw,
+    k_scale_pm_a(const u64* X, u64* Z, int n, int logN, int b, const ulonglong2* __restrict__ xtw,
                  const __grid_constant__ SumTab<NS, NS + 1> tq, const __grid_constant__ SumTab<NS + 1, NS> tb) {
     pdl_begin();
     constexpr int KS = NS + 1, LK = NS + KS;
@@ -316,17 +316,20 @@ __global__ void __launch_bounds__(256, 2)
             zo[0] = Z_EXACT;
             continue;
         }
+        u64 next = d[(size_t)NS << logN];   // a word ahead: a load does not pass the store of the word before it
 #pragma unroll
         for (int j = 0; j < KS; ++j) {
             const size_t l = (size_t)(NS + j) << logN;
-            zo[(size_t)j << logN] = scale_term<NS>(d[l], __ldg(f + l), g, v, tq, j, b);
+            const u64 w = next;
+            if (j + 1 < KS) next = d[(size_t)(NS + j + 1) << logN];
+            zo[(size_t)j << logN] = scale_term<NS>(w, __ldg(f + l), g, v, tq, j, b);
         }
     }
 }
 
 template <int NS>
 __global__ void __launch_bounds__(256, 2)
-    k_scale_pm_b(const u64* __restrict__ X, const u64* __restrict__ Z, u64* __restrict__ C3, int n, int logN, int b,
+    k_scale_pm_b(const u64* X, const u64* Z, u64* C3, int n, int logN, int b,
                  const __grid_constant__ SumTab<NS + 1, NS> tb, const __grid_constant__ ExactScale ex) {
     pdl_begin();
     constexpr int KS = NS + 1, LK = NS + KS;
@@ -378,7 +381,7 @@ __device__ __noinline__ u64 dec_exact(const u64* V, const u64* c0, int N, ExtDes
 
 template <int NS>
 __global__ void __launch_bounds__(256, 4)
-    k_dec_pm(const u64* __restrict__ V, const u64* __restrict__ ct, u64* __restrict__ M, int n, int logN, int b, ExtDesc ext,
+    k_dec_pm(const u64* V, const u64* ct, u64* M, int n, int logN, int b, ExtDesc ext,
              const u64* tmod, int nP, uint32_t* flags, const __grid_constant__ DecTab<NS> p) {
     pdl_begin();
     const int k = b - 28, hs = (b + 2) >> 1;

@@ -324,7 +324,7 @@ __global__ void __launch_bounds__(256, 2) k_inner(const u64* Dg, const u64* rlk,
 // Montgomery's reduction was bound by the multiplier pipe (97%): 28 instead of 42 multiplies per output at L = 8, where
 // it now waits on its digit loads (64 ciphertexts at N = 16384: 172 -> 158 us, 5.4 TB/s).
 template <int L>
-__global__ void __launch_bounds__(256, 2) k_inner_pm(const u64* __restrict__ Dg, const u64* __restrict__ rlk, u64* __restrict__ W,
+__global__ void __launch_bounds__(256, 2) k_inner_pm(const u64* Dg, const u64* rlk, u64* W,
                                                      int n, int QP, int cpg, PrimeTab tab, int logN, int b) {
     pdl_begin();
     constexpr bool KARA = L <= 8;
@@ -345,7 +345,7 @@ __global__ void __launch_bounds__(256, 2) k_inner_pm(const u64* __restrict__ Dg,
         for (int j = 0; j < L; ++j)
 #pragma unroll
             for (int m = 0; m < 2; ++m) {
-                const u64 y = __ldg(rlk + ((size_t)j * 2 + m) * plane + off);
+                const u64 y = rlk[((size_t)j * 2 + m) * plane + off];
                 yl[m][j] = (uint32_t)y & mask;
                 yh[m][j] = (uint32_t)(y >> hs);
                 if constexpr (KARA) ys[m][j] = yl[m][j] + yh[m][j];
