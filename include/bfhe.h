@@ -109,6 +109,13 @@ int bfhe_check(bfhe_ctx* ctx, void* stream, uint32_t* flags_out);
  * growth, hence device synchronisation, inside later calls). */
 int bfhe_reserve(bfhe_ctx* ctx, size_t n);
 
+/* How often the scratch arena has been (re)allocated; 0 for a NULL context.
+ * Calls recorded in a CUDA graph hold the arena's address, and a call that
+ * needs more scratch than the context has frees the arena and allocates a
+ * larger one.  A recorded graph may be replayed while this returns what it
+ * returned when the recording ended; afterwards it must be recorded again. */
+uint64_t bfhe_scratch_generation(const bfhe_ctx* ctx);
+
 /* Device memory the context holds, in bytes (host buffer of 4): out[0] the
  * constant tables (moduli, twiddles, twists, extension tables), out[1] the
  * keys (0 before keygen), out[2] the scratch arena (it grows to the largest
@@ -263,7 +270,8 @@ int bfhe_bit_gate(bfhe_ctx* ctx, int gate, const uint64_t* x, const uint64_t* y,
  * wire that another entry of the same call writes; wire indices must be
  * < n_wires (not checked on the device).  Counts only the multiplies.
  * Needs no host synchronisation: capturable in a CUDA graph once scratch is
- * reserved (bfhe_reserve) and one call of the same shape has run. */
+ * reserved (bfhe_reserve) and one call of the same shape has run; a recorded
+ * graph stays valid as bfhe_scratch_generation says. */
 enum { BFHE_OP_MUL = 8, BFHE_OP_LIN = 9 };
 int bfhe_gate_level(bfhe_ctx* ctx, uint64_t* wires, size_t n_wires, size_t n, const int32_t* table,
                     size_t n_gates, size_t n_mul, void* stream);

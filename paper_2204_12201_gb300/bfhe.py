@@ -45,6 +45,7 @@ def load():
         "bfhe_reserve": (I, [P, S]),
         "bfhe_ctx_device_bytes": (I, [P, P]),
         "bfhe_mul_scratch_bytes": (S, [P, S]),
+        "bfhe_scratch_generation": (U64, [P]),
         "bfhe_keygen": (I, [P, U64, P]),
         "bfhe_export_keys": (I, [P, P, P, P, P]),
         "bfhe_encrypt": (I, [P, P, S, U64, P, P]),
@@ -211,6 +212,11 @@ class Context:
         out = (ctypes.c_size_t * 4)()
         _check(self.lib.bfhe_ctx_device_bytes(self.h, out))
         return {"tables": out[0], "keys": out[1], "scratch": out[2], "other": out[3]}
+
+    @property
+    def scratch_generation(self):
+        """Changes when a call had to move the scratch arena: CUDA graphs recorded before then must not be replayed."""
+        return self.lib.bfhe_scratch_generation(self.h)
 
     def mul_scratch_bytes(self, n):
         """Scratch one mul_relin of n ciphertexts uses."""

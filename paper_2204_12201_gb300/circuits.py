@@ -259,6 +259,7 @@ class Compiled:
         self.depth = sum(1 for _, muls, _ in net.schedule() if muls)
         self.wires = torch.zeros(net.n_wires, n, 2, ctx.L, ctx.N, dtype=torch.int64, device=ctx.device)
         self.graph = None
+        self.generation = None   # the context's scratch arena that the graph's kernels work in
 
     def _table(self, rows, n_mul):
         t = torch.tensor(rows, dtype=torch.int32, device=self.ctx.device)
@@ -283,10 +284,13 @@ class Compiled:
             with torch.cuda.graph(g, stream=s):
                 self.run()
         torch.cuda.current_stream(self.ctx.device).wait_stream(s)
-        self.graph = g
+        self.graph, self.generation = g, self.ctx.scratch_generation
         return g
 
     def replay(self):
+        """Run the recorded graph; records it again when a larger call on the context has moved the scratch arena."""
+        if self.graph is not None and self.ctx.scratch_generation != self.generation:
+            self.capture()
         self.graph.replay()
 
     def out(self, wire_ids):

@@ -334,6 +334,7 @@ struct bfhe_ctx {
     // scratch
     void* scratch = nullptr;
     size_t scratch_bytes = 0;
+    uint64_t scratch_gen = 0;    // arenas so far: kernels recorded in a CUDA graph hold the address of one
     size_t reserve_n = 0;
 
     uint64_t counts[4] = {0, 0, 0, 0};

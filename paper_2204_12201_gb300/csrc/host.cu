@@ -408,6 +408,7 @@ int ctx_scratch(bfhe_ctx* ctx, size_t bytes, void** out) {
     if (ctx->scratch) BFHE_CUDA(cudaFree(ctx->scratch));
     ctx->scratch = nullptr;
     ctx->scratch_bytes = 0;
+    ++ctx->scratch_gen;
     const size_t want = (bytes + 255) & ~(size_t)255;
     cudaError_t e = cudaMalloc(&ctx->scratch, want);
     if (e != cudaSuccess) {
@@ -849,6 +850,8 @@ extern "C" int bfhe_ctx_device_bytes(const bfhe_ctx* ctx, size_t* out) {
     out[3] = ctx->d_cbase ? sizeof(u64) : 0;
     return BFHE_OK;
 }
+
+extern "C" uint64_t bfhe_scratch_generation(const bfhe_ctx* ctx) { return ctx ? ctx->scratch_gen : 0; }
 
 extern "C" size_t bfhe_mul_scratch_bytes(const bfhe_ctx* ctx, size_t n) { return ctx ? mul_scratch_bytes(ctx, n) : 0; }
 
