@@ -138,11 +138,12 @@ size_t bfhe_mul_scratch_bytes(const bfhe_ctx* ctx, size_t n);
  * below 2^50 and at most 16 data primes (BFHE_EINVAL otherwise).  Default: on
  * from 8 to 16 data primes (where it measured faster on GB300), off
  * otherwise.  With moduli of 45 to 55 bits and at most 16 data primes another
- * guarded form of the same conversion runs whatever the default, unless the
- * extension has been switched off by this call (then mixed radix alone).  bfhe_fast_extension
- * returns the current setting (1 or 0; BFHE_EINVAL for a NULL context).  The
- * paper has no counterpart: SEAL, which it runs on, uses approximate fast
- * conversions of this family. */
+ * guarded form of the same conversion runs, with the setting on and also where
+ * it is off by default; it gives way to mixed radix when this call switches
+ * off a setting that is on by default.  bfhe_fast_extension returns the
+ * current setting (1 or 0; BFHE_EINVAL for a NULL context); setting what it
+ * returned restores the context's state.  The paper has no counterpart: SEAL,
+ * which it runs on, uses approximate fast conversions of this family. */
 int bfhe_set_fast_extension(bfhe_ctx* ctx, int on);
 int bfhe_fast_extension(const bfhe_ctx* ctx);
 

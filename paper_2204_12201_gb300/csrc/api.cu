@@ -200,7 +200,8 @@ extern "C" int bfhe_set_fast_extension(bfhe_ctx* c, int on) {
     if (on && c->L > BFHE_MAX_L_UNROLLED)
         return set_error(BFHE_EINVAL, "the fast extension is built for at most 16 data primes");
     c->fast_ext = on != 0;
-    c->exact_ext = on == 0;
+    // where the default is off, off is the context as it was made: writing back what was read changes nothing
+    c->exact_ext = !on && c->fast_default;
     return BFHE_OK;
 }
 

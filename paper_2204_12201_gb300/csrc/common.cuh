@@ -339,7 +339,8 @@ struct bfhe_ctx {
 
     uint64_t counts[4] = {0, 0, 0, 0};
     bool fast_ext = false;       // guarded fast base extension in the multiply (bfhe_set_fast_extension)
-    bool exact_ext = false;      // the caller has switched it off: mixed radix everywhere
+    bool fast_default = false;   // its setting when the context is made
+    bool exact_ext = false;      // the caller has switched off a setting that is on by default: mixed radix everywhere
     bool pm_ext = false;         // the extensions of ext_pm.cu are available (at most 16 primes, pm)
     bool use_pm_ext() const { return pm_ext && !exact_ext; }
 

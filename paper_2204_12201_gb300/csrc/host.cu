@@ -804,9 +804,10 @@ extern "C" int bfhe_ctx_create(const bfhe_params* prm, int device, bfhe_ctx** ou
     }
     // the guarded fast extension of ext.cu measures faster from 8 data primes up (slower at 2); that of ext_pm.cu, for
     // moduli 2^b - d, at every size (64 pairs, lift + scale-and-round: N = 4096, L = 2: 61 -> 43 us, N = 8192, L = 4:
-    // 242 -> 138), so it also replaces the mixed-radix path where the setting is off by default
+    // 242 -> 138), so it also replaces the mixed-radix path where the setting is off by
+    // default, and stays there (bfhe_set_fast_extension)
     c->pm_ext = pm_ext;
-    c->fast_ext = c->L >= 8 && c->L <= BFHE_MAX_L_UNROLLED && c->ext_QB.fast_ok && c->ext_BQ.fast_ok;
+    c->fast_default = c->fast_ext = c->L >= 8 && c->L <= BFHE_MAX_L_UNROLLED && c->ext_QB.fast_ok && c->ext_BQ.fast_ok;
     c->d_tmod = base + o_tmod;
     c->d_delta_q = base + o_delta;
     c->d_Qinv_b = base + o_Qinvb;
