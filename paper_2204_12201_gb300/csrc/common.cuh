@@ -488,4 +488,5 @@ int launch_ntt_fwd(const bfhe_ctx* ctx, NttIO io, int n_polys, int n_limbs, Limb
 // below q) for consumers that fold the twist into a product of their own (scale-and-round, mod-down)
 int launch_ntt_inv(const bfhe_ctx* ctx, NttIO io, int n_polys, int n_limbs, LimbMap map, int mont,
                    cudaStream_t st, int lazy_out = 0);
-int ntt_config(int logN, int inverse, size_t limbs, int* log_m, int* log_e);   // shape of a launch of `limbs` limbs
+// shape of a launch of `limbs` limbs; pm: products modulo 2^b - d
+int ntt_config(int logN, int inverse, bool pm, size_t limbs, int* log_m, int* log_e);

@@ -585,15 +585,18 @@ int env_int(const char* name) {
 // as two 16384-word halves, 32 words (8 pairs, L = 16: 887 / 347; 16 words 949 / 471).  A launch whose halves fit the 152
 // SMs at one CTA each takes halves at 16 words, which puts twice the threads on each limb: at N = 16384 (72 limbs: 14 / 15
 // against 19 / 19) and for the forward at N = 8192 (8.3 against 12.5); the inverse there takes one block of 16 words
-// (up to 152 limbs: 10.4 to 11.7 against 12.4; halves 10.3).  bfhe_ntt_config (the autotuner) or BFHE_NTT_LOG_M /
+// (up to 152 limbs: 10.4 to 11.7 against 12.4; halves 10.3).  The Shoup products' kernels take the same shapes (64 pairs
+// at N = 8192, L = 4, 40 bits: 219 / 162, 16 words 266 / 193) but for the forward at N = 16384, in halves of 32 words (64
+// pairs, L = 8: 1139 against 1188 us at 40 bits, 1301 against 1358 at 56).  bfhe_ntt_config (the autotuner) or BFHE_NTT_LOG_M /
 // BFHE_NTT_LOG_E override the defaults.
 int g_cfg[16][2][2] = {};   // [logN][inverse] -> (log_m, log_e), 0 = default
 
-int ntt_config(int logN, int inverse, size_t limbs, int* log_m, int* log_e) {
+int ntt_config(int logN, int inverse, bool pm, size_t limbs, int* log_m, int* log_e) {
     static const int env_m = env_int("BFHE_NTT_LOG_M");
     static const int env_e = env_int("BFHE_NTT_LOG_E");
     int m = logN <= 14 ? logN : logN - 1;
     int e = logN >= 13 ? 5 : 4;
+    if (logN == 14 && !inverse && !pm) m = 13;
     if ((logN == 14 || (logN == 13 && !inverse)) && 2 * limbs <= 152) {
         m = logN - 1;
         e = 4;
@@ -622,7 +625,7 @@ extern "C" int bfhe_ntt_config(uint32_t logN, int inverse, uint32_t log_m, uint3
         g_cfg[logN][inverse ? 1 : 0][1] = (int)log_e;
     }
     int m, e;
-    ntt_config((int)logN, inverse, (size_t)1 << 30, &m, &e);   // the shape of a large launch
+    ntt_config((int)logN, inverse, true, (size_t)1 << 30, &m, &e);   // the shape of a large launch of the default moduli
     if (cur_m) *cur_m = (uint32_t)m;
     if (cur_e) *cur_e = (uint32_t)e;
     return BFHE_OK;
@@ -633,10 +636,10 @@ int launch_ntt_fwd(const bfhe_ctx* ctx, NttIO io, int n_polys, int n_limbs, Limb
     if (n_polys <= 0 || n_limbs <= 0) return BFHE_OK;
     ProfScope ps(ctx, BFHE_K_NTT_FWD, st, (double)n_polys * n_limbs * (ctx->N / 2) * ctx->logN,
                  16.0 * n_polys * n_limbs * ctx->N);
-    int log_m, log_e;
-    ntt_config((int)ctx->logN, 0, (size_t)n_polys * n_limbs, &log_m, &log_e);
     // the slot modulus t (prime index nP - 1) is not of the form 2^b - d
     const bool pm = ctx->pm && map(0) != (int)ctx->nP - 1;
+    int log_m, log_e;
+    ntt_config((int)ctx->logN, 0, pm, (size_t)n_polys * n_limbs, &log_m, &log_e);
     NttArgs a = make_args(ctx, io, n_limbs, map, 0, lazy_out && (pm || ctx->prime_bits <= 50) ? 1 : 0);
     const int blocks = n_polys * n_limbs;
     const int subs = (int)(ctx->N >> log_m);
@@ -650,14 +653,14 @@ int launch_ntt_inv(const bfhe_ctx* ctx, NttIO io, int n_polys, int n_limbs, Limb
     if (n_polys <= 0 || n_limbs <= 0) return BFHE_OK;
     ProfScope ps(ctx, BFHE_K_NTT_INV, st, (double)n_polys * n_limbs * (ctx->N / 2) * ctx->logN,
                  16.0 * n_polys * n_limbs * ctx->N);
+    const bool pm = ctx->pm && map(0) != (int)ctx->nP - 1;
     int log_m, log_e;
-    ntt_config((int)ctx->logN, 1, (size_t)n_polys * n_limbs, &log_m, &log_e);
+    ntt_config((int)ctx->logN, 1, pm, (size_t)n_polys * n_limbs, &log_m, &log_e);
     NttArgs a = make_args(ctx, io, n_limbs, map, mont, lazy_out);
     const int blocks = n_polys * n_limbs;
     const int subs = (int)(ctx->N >> log_m);
     if (subs != 1 && subs != 2) return set_error(BFHE_EINVAL, "unsupported ring degree");
     if (lazy_out != 0 && lazy_out != 2) return set_error(BFHE_EINVAL, "bad inverse output form");
-    const bool pm = ctx->pm && map(0) != (int)ctx->nP - 1;
     if (io.mul) {
         if (!pm || lazy_out) return set_error(BFHE_EINVAL, "the inverse of a product needs moduli 2^b - d");
         return ntt_inv_mul_any_pm(a, log_m, log_e, blocks, subs == 2, st);
