@@ -161,11 +161,15 @@ __global__ void __launch_bounds__(256, NS <= 8 ? 4 : 2) k_modup(const u64* A, co
 
 // scale-and-round of the tensor (X slots 0..2, Q u B limbs) into C3 [n][3][L][N].  The inverse transforms
 // leave the tensor untwisted: the first product of each limb, by t, also carries the twist N^-1 psi^-k R.
-template <int NS, int KS, bool FAST>
+// PM: moduli 2^bits - d (mixed radix alone, where the caller has switched the guarded form off); a choice at run time
+// between the two products costs every instance 10 to 20% (64 pairs at N = 16384, L = 8: 613 -> 717 us at 40 bits, 860 -> 940 at 56).
+template <int NS, int KS, bool FAST, bool PM>
 __global__ void __launch_bounds__(256, 2) k_scale(const u64* X, u64* C3, int n, ExtDesc eQB, ExtDesc eBQ, const u64* twist, int nP,
                         const u64* Qinv_b, const u64* bq, int N, int bits, FastTab<FAST ? NS : 1, FAST ? KS : 1> fq,
                         FastTab<FAST ? KS : 1, FAST ? NS : 1> fb) {
     pdl_begin();
+    static_assert(!(FAST && PM), "moduli 2^b - d have a guarded form of their own");
+    if (!PM) bits = 0;
     const size_t total = (size_t)n * 3 * N;
     constexpr int LK = NS + KS;
     for (size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
@@ -229,7 +233,7 @@ __global__ void __launch_bounds__(256, 2) k_scale(const u64* X, u64* C3, int n, 
 // Measured at N = 32768, L = 16: mul_relin +10.6%, squarings +12.1%; at L = 8 the one-pass kernel is 1% faster.
 template <int NS, int KS>
 __global__ void __launch_bounds__(256, 2) k_scale_a(const u64* X, u64* Yt, int n, ExtDesc eQB, const u64* twist, int nP,
-                                                    const u64* Qinv_b, const u64* bq, int N, int bits, FastTab<NS, KS> fq) {
+                                                    const u64* Qinv_b, const u64* bq, int N, FastTab<NS, KS> fq) {
     pdl_begin();
     const size_t total = (size_t)n * 3 * N;
     constexpr int LK = NS + KS;
@@ -249,7 +253,7 @@ __global__ void __launch_bounds__(256, 2) k_scale_a(const u64* X, u64* Yt, int n
 #pragma unroll
             for (int i = 0; i < NS; ++i) {
                 const ulonglong2 f = twist_at(twist, i, 2, k, N);
-                r[i] = twist_mul(d[(size_t)i * N], f, eQB.src_q[i], bits);
+                r[i] = twist_mul(d[(size_t)i * N], f, eQB.src_q[i], 0);
             }
             fast = fast_prep<NS, KS>(r, eQB, fq, r0, r1, vv);
         }
@@ -259,14 +263,14 @@ __global__ void __launch_bounds__(256, 2) k_scale_a(const u64* X, u64* Yt, int n
 #pragma unroll
             for (int i = 0; i < NS; ++i) {
                 const ulonglong2 f = twist_at(twist, i, 2, k, N);
-                r[i] = twist_mul(d[(size_t)i * N], f, eQB.src_q[i], bits);
+                r[i] = twist_mul(d[(size_t)i * N], f, eQB.src_q[i], 0);
             }
             const bool neg = garner<NS>(r, eQB, v);
             for (int j = 0; j < KS; ++j) {
                 const u64 bj = bq[j];
                 const int pj = NS + (nP - 1 - NS - KS) + j;
                 const ulonglong2 f = twist_at(twist, pj, 2, k, N);
-                const u64 td = twist_mul(d[(size_t)(NS + j) * N], f, bj, bits);
+                const u64 td = twist_mul(d[(size_t)(NS + j) * N], f, bj, 0);
                 const u64 rb = ext_eval<NS, false>(v, neg, eQB, j);
                 yo[(size_t)j * N] = shoup_lazy(td + bj - rb, Qinv_b[j], Qinv_b[KS + j], bj);
             }
@@ -277,7 +281,7 @@ __global__ void __launch_bounds__(256, 2) k_scale_a(const u64* X, u64* Yt, int n
             const u64 bj = bq[j];
             const int pj = NS + (nP - 1 - NS - KS) + j;
             const ulonglong2 f = twist_at(twist, pj, 2, k, N);
-            const u64 td = twist_mul(d[(size_t)(NS + j) * N], f, bj, bits);
+            const u64 td = twist_mul(d[(size_t)(NS + j) * N], f, bj, 0);
             const u64 rb = fast_eval3<NS, KS>(r0, r1, vv, eQB, fq, j);
             yo[(size_t)j * N] = shoup_lazy(td + bj - rb, Qinv_b[j], Qinv_b[KS + j], bj);
         }
@@ -591,23 +595,31 @@ template <int NS>
 int run_scale(const bfhe_ctx* ctx, const u64* X, u64* C3, int n, cudaStream_t st, u64* tmp) {
     const size_t work = (size_t)n * 3 * ctx->N;
     const u64* bq = ctx->tab.q + ctx->L + ctx->alpha;
+    if (ctx->pm) {   // the extension switched off, which is possible where it is on by default
+        if constexpr (NS >= 8) {
+            LAUNCH((k_scale<NS, NS + 1, false, true>), work, X, C3, n, ctx->ext_QB, ctx->ext_BQ, ctx->tab.twist, (int)ctx->nP,
+                   ctx->d_Qinv_b, bq, (int)ctx->N, ctx->pm_bits(), FastTab<1, 1>{}, FastTab<1, 1>{});
+            return BFHE_OK;
+        }
+        return set_error(BFHE_EINVAL, "no mixed-radix scale-and-round for these moduli");
+    }
     const bool fast = ctx->fast_ext && ctx->ext_QB.fast_ok && ctx->ext_BQ.fast_ok;
     if constexpr (NS >= 10) {
         if (tmp && fast) {
             LAUNCH((k_scale_a<NS, NS + 1>), work, X, tmp, n, ctx->ext_QB, ctx->tab.twist, (int)ctx->nP,
-                   ctx->d_Qinv_b, bq, (int)ctx->N, ctx->pm_bits(), fast_tab<NS, NS + 1>(ctx->exth_QB));
+                   ctx->d_Qinv_b, bq, (int)ctx->N, fast_tab<NS, NS + 1>(ctx->exth_QB));
             LAUNCH((k_scale_b<NS, NS + 1>), work, tmp, C3, n, ctx->ext_BQ, (int)ctx->N,
                    fast_tab<NS + 1, NS>(ctx->exth_BQ));
             return BFHE_OK;
         }
     }
     if (fast)
-        LAUNCH((k_scale<NS, NS + 1, true>), work, X, C3, n, ctx->ext_QB, ctx->ext_BQ, ctx->tab.twist, (int)ctx->nP,
-               ctx->d_Qinv_b, bq, (int)ctx->N, ctx->pm_bits(), fast_tab<NS, NS + 1>(ctx->exth_QB),
+        LAUNCH((k_scale<NS, NS + 1, true, false>), work, X, C3, n, ctx->ext_QB, ctx->ext_BQ, ctx->tab.twist, (int)ctx->nP,
+               ctx->d_Qinv_b, bq, (int)ctx->N, 0, fast_tab<NS, NS + 1>(ctx->exth_QB),
                fast_tab<NS + 1, NS>(ctx->exth_BQ));
     else
-        LAUNCH((k_scale<NS, NS + 1, false>), work, X, C3, n, ctx->ext_QB, ctx->ext_BQ, ctx->tab.twist, (int)ctx->nP,
-               ctx->d_Qinv_b, bq, (int)ctx->N, ctx->pm_bits(), FastTab<1, 1>{}, FastTab<1, 1>{});
+        LAUNCH((k_scale<NS, NS + 1, false, false>), work, X, C3, n, ctx->ext_QB, ctx->ext_BQ, ctx->tab.twist, (int)ctx->nP,
+               ctx->d_Qinv_b, bq, (int)ctx->N, 0, FastTab<1, 1>{}, FastTab<1, 1>{});
     return BFHE_OK;
 }
 
