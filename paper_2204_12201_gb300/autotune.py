@@ -50,6 +50,14 @@ def _best_ms(torch, fn, reps=3):
     return best
 
 
+def _pick(timings, now):
+    """The fastest pair, or the one in use when it is within 1% of it: repetitions differ by that much, and any pair but
+    the built-in one replaces the library's rule for small launches too (a single product at N = 16384, L = 8: 76 us by the rule,
+    107 with its large launches' shape throughout)."""
+    best = min(timings, key=timings.get)
+    return now if timings.get(now, float("inf")) <= 1.01 * timings[best] else best
+
+
 def tune_ring(N, verbose=False):
     """Search one ring degree; returns {"fwd", "inv", "tile", "ms"} and installs the result."""
     import torch
@@ -63,13 +71,14 @@ def tune_ring(N, verbose=False):
     o = torch.empty_like(a)
     x, y, z = a[:B], b[:B], o[:B]
     bfhe.set_mul_tile(logN, 0)
+    now = "%d,%d/%d,%d" % (bfhe.ntt_config(logN, 0) + bfhe.ntt_config(logN, 1))
     timings = {}
     for fm, fe in shapes(logN):
         bfhe.ntt_config(logN, 0, fm, fe)
         for im, ie in shapes(logN):
             bfhe.ntt_config(logN, 1, im, ie)
             timings["%d,%d/%d,%d" % (fm, fe, im, ie)] = _best_ms(torch, lambda: ctx.mul_relin(x, y, out=z), reps=5)
-    best = min(timings, key=timings.get)
+    best = _pick(timings, now)
     fwd, inv = ([int(v) for v in part.split(",")] for part in best.split("/"))
     bfhe.ntt_config(logN, 0, *fwd)
     bfhe.ntt_config(logN, 1, *inv)

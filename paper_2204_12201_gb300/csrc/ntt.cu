@@ -621,8 +621,14 @@ extern "C" int bfhe_ntt_config(uint32_t logN, int inverse, uint32_t log_m, uint3
         if (log_m > logN || log_m + 1 < logN || log_m < 10 || log_m > 14 || log_e < 3 || log_e > 5 ||
             (log_m == 14 && log_e < 4))
             return set_error(BFHE_EINVAL, "unsupported NTT block configuration");
-        g_cfg[logN][inverse ? 1 : 0][0] = (int)log_m;
-        g_cfg[logN][inverse ? 1 : 0][1] = (int)log_e;
+        // the shape that large launches take anyway is no override: small launches keep theirs
+        int dm, de;
+        g_cfg[logN][inverse ? 1 : 0][0] = 0;
+        ntt_config((int)logN, inverse, true, (size_t)1 << 30, &dm, &de);
+        if ((int)log_m != dm || (int)log_e != de) {
+            g_cfg[logN][inverse ? 1 : 0][0] = (int)log_m;
+            g_cfg[logN][inverse ? 1 : 0][1] = (int)log_e;
+        }
     }
     int m, e;
     ntt_config((int)logN, inverse, true, (size_t)1 << 30, &m, &e);   // the shape of a large launch of the default moduli
