@@ -137,7 +137,8 @@ size_t bfhe_mul_scratch_bytes(const bfhe_ctx* ctx, size_t n);
  * either way (bit for bit); only the speed differs.  Needs every modulus
  * below 2^50 and at most 16 data primes (BFHE_EINVAL otherwise).  Default: on
  * from 8 to 16 data primes (where it measured faster on GB300), off
- * otherwise.  With moduli of 45 to 55 bits and at most 16 data primes another
+ * otherwise.  With moduli of 45 to 55 bits and at most 16 data primes (but not
+ * at 55 bits, N = 32768 and more than 10 data primes, 9 with alpha = 2) another
  * guarded form of the same conversion runs, with the setting on and also where
  * it is off by default; it gives way to mixed radix when this call switches
  * off a setting that is on by default.  bfhe_fast_extension returns the

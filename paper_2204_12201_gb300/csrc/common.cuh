@@ -376,6 +376,7 @@ struct bfhe_ctx {
 };
 
 // ------------------------------------------------------------------ host helpers (host.cu)
+bool pm_bounded(uint32_t bits, uint32_t logN, u64 d);   // bfhe_ctx::pm of moduli 2^bits - d at ring degree 2^logN
 int set_error(int code, const std::string& msg);
 // process-wide count of kernel launches made by this library (measurement)
 void count_launch();

@@ -505,6 +505,17 @@ extern "C" int bfhe_param_primes(const bfhe_params* prm, uint64_t* primes_out, u
     return BFHE_OK;
 }
 
+// Products as pm_mul (common.cuh) when every transform stays below 2^63 in magnitude, d the largest 2^bits - q: one stage
+// adds at most 3 2^29 4d + 2.5 2^(bits + 2); the forward starts below 2^60 (the lift's sums, 2^(bits + 1) above 52 bits),
+// the inverse's first pass sums up to 32 inputs (below 2^bits + 2^(63 - bits) d each).  With 45 to 55 bits it fails where
+// d is large and many stages add to it: at 55 bits for N = 32768 from 11 data primes (10 with two special primes) and
+// N = 16384 from 29 (28), at 54 bits for N = 32768 from 22 (21).
+bool pm_bounded(uint32_t bits, uint32_t logN, u64 d) {
+    if (bits < 45 || bits > 55) return false;
+    const u128 g = (u128)6442450944ull * d + ((u128)5 << (bits + 1));
+    return (u128)logN * g + ((u128)1 << (bits > 52 ? bits + 5 : 60)) + ((u128)1 << 45) < ((u128)1 << 63);
+}
+
 extern "C" int bfhe_ctx_create(const bfhe_params* prm, int device, bfhe_ctx** out) {
     if (!prm || !out) return set_error(BFHE_EINVAL, "null argument");
     *out = nullptr;
@@ -532,14 +543,10 @@ extern "C" int bfhe_ctx_create(const bfhe_params* prm, int device, bfhe_ctx** ou
     c->nP = (uint32_t)c->primes.size();
     const uint32_t L = c->L, A = c->alpha, nP = c->nP;
 
-    // Products as pm_mul (common.cuh) when every transform stays below 2^63 in magnitude: one stage adds at most
-    // 3 2^29 4d + 2.5 2^(bits + 2); the forward starts below 2^60 (the lift's sums, 2^(bits + 1) above 52 bits), the
-    // inverse's first pass sums up to 32 inputs (below 2^bits + 2^(63 - bits) d each).
-    if (bits >= 45 && bits <= 55) {
+    {
         u64 d = 0;
         for (u64 q : rule.moduli) d = std::max(d, ((u64)1 << bits) - q);
-        const u128 g = (u128)6442450944ull * d + ((u128)5 << (bits + 1));
-        c->pm = (u128)c->logN * g + ((u128)1 << (bits > 52 ? bits + 5 : 60)) + ((u128)1 << 45) < ((u128)1 << 63);
+        c->pm = pm_bounded(bits, c->logN, d);
     }
     // bit reversal
     c->brv.resize(N);
