@@ -52,16 +52,10 @@ __host__ __device__ __forceinline__ u64 shoup_lazy(u64 a, u64 w, u64 ws, u64 q) 
 // a * w mod q in [0, 4q) for a < 2^64: the quotient estimate keeps a1 w1 and the high
 // halves of the two cross products a1 w0, a0 w1 (their low halves and a0 w0 together are
 // below 3 2^64), so it is floor(a ws / 2^64) minus 0, 1 or 2, and Shoup's own estimate
-// is the true quotient or one less.
-__host__ __device__ __forceinline__ u64 shoup_lazy4(u64 a, u64 w, u64 ws, u64 q) {
-    const uint32_t a0 = (uint32_t)a, a1 = (uint32_t)(a >> 32), w0 = (uint32_t)ws, w1 = (uint32_t)(ws >> 32);
-    const u64 hi = (u64)a1 * w1 + (((u64)a1 * w0) >> 32) + (((u64)a0 * w1) >> 32);
-    return a * w - hi * q;
-}
-
-// The same product with the modulus passed negated (nq = 2^64 - q): r = a w + h nq mod 2^64, written
-// in 32-bit pieces so that each partial product is one multiply-add (the low word of a0 w0 + h0 nq0 as
-// one wide multiply-add, the high word as four narrow ones).
+// is the true quotient or one less.  The modulus is passed negated (nq = 2^64 - q):
+// r = a w + h nq mod 2^64, written in 32-bit pieces so that each partial product is one
+// multiply-add (the low word of a0 w0 + h0 nq0 as one wide multiply-add, the high word as
+// four narrow ones).
 __device__ __forceinline__ u64 shoup_lazy4n(u64 a, u64 w, u64 ws, u64 nq) {
     const uint32_t a0 = (uint32_t)a, a1 = (uint32_t)(a >> 32), s0 = (uint32_t)ws, s1 = (uint32_t)(ws >> 32);
     u64 h = (u64)a1 * s1 + __umulhi(a1, s0);
